@@ -181,7 +181,9 @@ int lbm_porosity_errors(lbm_handle *h, uint32_t *count, int clear);
  * step count. */
 int lbm_init_fields(lbm_handle *h, const float *ur, const float *uz, const float *T, int on_device);
 
-/* Advance nsteps >= 0 time steps (asynchronous on the handle's stream). */
+/* Advance nsteps >= 0 time steps (asynchronous on the handle's stream).  With FP32 storage
+ * in two buffers (and no discrete heater) pairs of steps share a launch; the last step of a
+ * call is always a launch of its own, so that the previous state is kept (lbm_residual). */
 int lbm_step(lbm_handle *h, int64_t nsteps);
 
 /* Fields of the current state (what the next step's pull sees, after the wall
@@ -307,7 +309,8 @@ int lbm_set_staging(lbm_handle *h, int enable);
 /* Per-launch timing of the step kernels with CUDA events on the handle's stream.
  * enable = 1 starts recording (and clears the totals), 0 stops.  lbm_kernel_times
  * synchronises and returns the summed milliseconds and launch counts of the bulk
- * step kernel and of the wall-node kernel since timing was enabled. */
+ * step kernel and of the wall-node kernel since timing was enabled (a launch of two steps
+ * counts as one bulk launch; its boundary nodes are part of it). */
 int lbm_set_timing(lbm_handle *h, int enable);
 int lbm_kernel_times(lbm_handle *h, double *bulk_ms, int64_t *bulk_launches, double *wall_ms,
                      int64_t *wall_launches);

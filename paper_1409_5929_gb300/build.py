@@ -21,7 +21,8 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 TARGETS = {
     "liblbm.so": ([os.path.join(CSRC, "lbm.cu")],
-                  [os.path.join(CSRC, "lbm_physics.cuh"), os.path.join(INC, "lbm.h")]),
+                  [os.path.join(CSRC, n) for n in ("lbm_physics.cuh", "lbm_pair.cuh", "lbm_two.cuh")] +
+                  [os.path.join(INC, "lbm.h")]),
     "libfno.so": ([os.path.join(CSRC, "fno.cu")], [os.path.join(INC, "fno.h")]),
     "libfnonet.so": ([os.path.join(CSRC, "fno_net.cu")], [os.path.join(CSRC, "tc.cuh"), os.path.join(INC, "fno_net.h")]),
 }

@@ -86,6 +86,7 @@ struct RowC {
     float kT;      // tau_T / r
     float cs2r;    // c_s^2 / r
     float c2r;     // c_s^2 2 (tau - 1/2) / r
+    float c2rr;    // c_s^2 2 (tau - 1/2) / r^2
 };
 
 __device__ __forceinline__ RowC row_consts(const Consts<float>& c, int kr) {
@@ -99,6 +100,7 @@ __device__ __forceinline__ RowC row_consts(const Consts<float>& c, int kr) {
     q.kT = c.tauT * q.inv_r;
     q.cs2r = cs2<float>() * q.inv_r;
     q.c2r = c.cs2_2tm * q.inv_r;
+    q.c2rr = q.c2r * q.inv_r;
     return q;
 }
 
