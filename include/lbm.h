@@ -182,8 +182,9 @@ int lbm_porosity_errors(lbm_handle *h, uint32_t *count, int clear);
 int lbm_init_fields(lbm_handle *h, const float *ur, const float *uz, const float *T, int on_device);
 
 /* Advance nsteps >= 0 time steps (asynchronous on the handle's stream).  With FP32 storage
- * in two buffers (and no discrete heater) pairs of steps share a launch; the last step of a
- * call is always a launch of its own, so that the previous state is kept (lbm_residual). */
+ * in two buffers (and no discrete heater) a launch holds the boundary nodes too, and on small
+ * and on large grids several steps; the last step of a call is always a launch of its own, so
+ * that the previous state is kept (lbm_residual). */
 int lbm_step(lbm_handle *h, int64_t nsteps);
 
 /* Fields of the current state (what the next step's pull sees, after the wall
@@ -309,8 +310,8 @@ int lbm_set_staging(lbm_handle *h, int enable);
 /* Per-launch timing of the step kernels with CUDA events on the handle's stream.
  * enable = 1 starts recording (and clears the totals), 0 stops.  lbm_kernel_times
  * synchronises and returns the summed milliseconds and launch counts of the bulk
- * step kernel and of the wall-node kernel since timing was enabled (a launch of two steps
- * counts as one bulk launch; its boundary nodes are part of it). */
+ * step kernel and of the wall-node kernel since timing was enabled (a launch that
+ * holds its boundary nodes, or several steps, counts as one bulk launch and no wall launch). */
 int lbm_set_timing(lbm_handle *h, int enable);
 int lbm_kernel_times(lbm_handle *h, double *bulk_ms, int64_t *bulk_launches, double *wall_ms,
                      int64_t *wall_launches);
@@ -363,7 +364,7 @@ int lbm_batch_set_porosity(lbm_batch *b, int32_t i, const float *phi, int on_dev
 /* (Re)initialise instance i as lbm_init_fields does; a stopped instance becomes
  * active again. */
 int lbm_batch_init_fields(lbm_batch *b, int32_t i, const float *ur, const float *uz, const float *T, int on_device);
-/* nsteps steps of every active instance (two launches per step for the whole batch). */
+/* nsteps steps of every active instance (one or two launches per step for the whole batch). */
 int lbm_batch_step(lbm_batch *b, int64_t nsteps);
 /* Step until every instance is steady (criterion of lbm_run, per instance, checked
  * every check_every steps; check_every must be even) or max_steps.  The steps of one

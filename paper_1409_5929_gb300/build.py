@@ -20,9 +20,9 @@ INC = os.path.join(ROOT, "include")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 TARGETS = {
-    "liblbm.so": ([os.path.join(CSRC, "lbm.cu")],
-                  [os.path.join(CSRC, n) for n in ("lbm_physics.cuh", "lbm_pair.cuh", "lbm_two.cuh")] +
-                  [os.path.join(INC, "lbm.h")]),
+    "liblbm.so": ([os.path.join(CSRC, "lbm.cu"), os.path.join(CSRC, "lbm_f32.cu")],
+                  [os.path.join(CSRC, n) for n in ("lbm_physics.cuh", "lbm_pair.cuh", "lbm_f32.h", "lbm_two.cuh",
+                                                   "lbm_tile.cuh", "lbm_step32.cuh")] + [os.path.join(INC, "lbm.h")]),
     "libfno.so": ([os.path.join(CSRC, "fno.cu")], [os.path.join(INC, "fno.h")]),
     "libfnonet.so": ([os.path.join(CSRC, "fno_net.cu")], [os.path.join(CSRC, "tc.cuh"), os.path.join(INC, "fno_net.h")]),
 }
@@ -50,7 +50,7 @@ def _build_one(name: str, force: bool, verbose: bool) -> str:
     if not force and not _stale(out, sources + headers):
         return out
     tmp = out + f".tmp{os.getpid()}"
-    cmd = [nvcc(), *ARCH, "-O3", "-lineinfo", "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I", INC,
+    cmd = [nvcc(), *ARCH, "-O3", "-lineinfo", "-std=c++17", "--threads", "4", "-shared", "-Xcompiler", "-fPIC", "-I", INC,
            "-o", tmp, *sources]
     if verbose:
         cmd.insert(1, "-Xptxas=-v")

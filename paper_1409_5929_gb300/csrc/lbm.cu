@@ -37,6 +37,7 @@
 #include <vector>
 
 #include "../../include/lbm.h"
+#include "lbm_f32.h"
 #include "lbm_pair.cuh"
 #include "lbm_physics.cuh"
 
@@ -826,74 +827,6 @@ static cudaError_t stage_carveout() {
     return e;
 }
 
-#include "lbm_two.cuh"
-
-// Two steps per pass (lbm_two.cuh): one warp per strip of columns and chunk of rows; warps are
-// independent.  At 4096 x 8192 a pass takes 0.68 ms for two steps where two single steps take
-// 1.24 ms (0.60 ms each, 97 % of the copy bandwidth, and the wall kernel): it moves the state's
-// 118 bytes per node once, at 86 % of the copy bandwidth, and issues 260 instructions per node
-// and step (563 in k_bulk).  128 registers, four blocks per SM; with five the registers spill
-// (0.44 ms per step), with three too few warps are in flight (0.40).  The marches that meet boundary nodes (the end strips, the first and the last
-// chunk of every strip, the wall rows) come first and run a form of the march of their own: the
-// boundary rebuild between a row's recovery and its collision cost the other marches 13 %
-// (4096 x 8192, FP32) when one form served both.
-#ifndef LBM_TWO_MIN_BLOCKS
-#define LBM_TWO_MIN_BLOCKS 4
-#endif
-// A march with boundary nodes takes about 1.6 times as long per row, so those get fewer rows.
-struct TwoPlan {
-    int strips, first, last;   // strips of columns; rows first .. last are pulled by second steps
-    int rows, erows;           // rows of a march without and with boundary nodes
-    __host__ __device__ int ends() const { return min(strips, 2); }
-    __host__ __device__ int inner() const { return strips - ends(); }
-    // end strips: all rows in chunks of erows; inner strips: the first and the last erows rows,
-    // and between them chunks of rows
-    __host__ __device__ int echunks() const { return (last - first + erows) / erows; }
-    __host__ __device__ int outer() const { return min(echunks(), 2); }
-    __host__ __device__ int mid() const { return max(last - first + 1 - 2 * erows, 0); }
-    __host__ __device__ int chunks() const { return (mid() + rows - 1) / rows; }
-    __host__ __device__ int walls() const { return 1 + first; }   // wall rows: 0 too unless it is a pipe axis
-    __host__ __device__ int n_wall() const { return strips * walls() + ends() * echunks() + inner() * outer(); }
-    __host__ __device__ int n_bulk() const { return inner() * chunks(); }
-};
-template <bool VEC>
-__global__ void __launch_bounds__(BULK_THREADS, LBM_TWO_MIN_BLOCKS) k_two(const Consts<float> c, const Buf<LBM_F32> A,
-                                                                         const Buf<LBM_F32> B,
-                                                                         const float* __restrict__ phi, int plane,
-                                                                         const TwoPlan w) {
-    __shared__ float4 ring[TWO_KEEP * BULK_THREADS];
-    constexpr int WARPS = BULK_THREADS / 32;
-    const int wall_blocks = (w.n_wall() + WARPS - 1) / WARPS, warp = threadIdx.x >> 5;
-    if ((int)blockIdx.x >= wall_blocks) {
-        const int t = ((int)blockIdx.x - wall_blocks) * WARPS + warp;
-        if (t >= w.n_bulk()) return;
-        const int chunk = t / w.inner(), lo = w.first + w.erows + chunk * w.rows;
-        two_march<VEC, false>(c, A, B, phi, plane, 1 + t - chunk * w.inner(), lo,
-                                   min(lo + w.rows - 1, w.last - w.erows), -1, ring);
-        return;
-    }
-    int t = blockIdx.x * WARPS + warp, s, lo, hi, wall = -1;
-    if (t < w.ends() * w.echunks()) {
-        const int chunk = t / w.ends();
-        s = t - chunk * w.ends() == 0 ? 0 : w.strips - 1;
-        lo = w.first + chunk * w.erows;
-        hi = min(lo + w.erows - 1, w.last);
-    } else if ((t -= w.ends() * w.echunks()) < w.inner() * w.outer()) {
-        const int chunk = t / w.inner();
-        s = 1 + t - chunk * w.inner();
-        lo = chunk == 0 ? w.first : max(w.last - w.erows + 1, w.first + w.erows);
-        hi = chunk == 0 ? min(w.first + w.erows - 1, w.last) : w.last;
-    } else {
-        t -= w.inner() * w.outer();
-        const int k = t / w.strips;
-        if (k >= w.walls()) return;
-        s = t - k * w.strips;
-        wall = k == 0 ? c.nr - 1 : 0;
-        lo = hi = wall ? w.last : 1;
-    }
-    two_march<VEC, true>(c, A, B, phi, plane, s, lo, hi, wall, ring);
-}
-
 // Wall nodes; LIN / LOUT: layouts read and written (in-place storage alternates S and L).
 template <int STO, int LIN = LAY_N, int LOUT = LAY_N>
 __global__ void k_wall(const Consts<float> c, const Buf<STO> A,
@@ -1500,7 +1433,8 @@ struct lbm_handle {
     int* wait_status = nullptr;    // 16-bit storage: LBM_ERR_TIMEOUT once a bounded wait of the staged kernel ran out
     int spin = STAGE_SPIN;         // try_wait rounds of its per-row waits
     int stage = 1;                 // 16-bit: the staged bulk kernel where it applies (lbm_set_staging)
-    TwoPlan two = {};              // marches of the two-step kernel (strips = 0: it does not serve this problem)
+    Plan32 plan = {};              // launches of several steps (FP32 storage, two buffers)
+    Consts32 c32;
 };
 
 static int derive(const lbm_params* p, lbm_info* o, Consts<double>* cd) {
@@ -1587,16 +1521,6 @@ static int derive(const lbm_params* p, lbm_info* o, Consts<double>* cd) {
         c.h_q = 1 - 0.5 * c.s_q;
         c.h_nu = 1 - 0.5 * c.s_nu;
         c.cs2_2tm = c.two_taum / 3.0;
-        c.a_e = c.s_e / 36;
-        c.g_u = c.s_e / 12;
-        c.g_f = c.h_e / 6;
-        c.a_j = c.s_j / 6;
-        c.b_j = c.h_j / 6;
-        c.a_q = c.s_q / 12;
-        c.b_q = c.h_q / 12;
-        c.a_nu = c.s_nu / 4;
-        c.b7 = c.h_nu / 2;
-        c.b8 = c.h_nu / 4;
         c.tauT = o->tau_T;
         c.wg_den = 1.0 / (o->tau_T + 0.5);
         c.gbeta = o->gbeta;
@@ -1636,8 +1560,6 @@ static Consts<float> to_float(const Consts<double>& d) {
     f.s_e = (float)d.s_e; f.s_eps = (float)d.s_eps; f.s_j = (float)d.s_j; f.s_q = (float)d.s_q; f.s_nu = (float)d.s_nu;
     f.h_e = (float)d.h_e; f.h_eps = (float)d.h_eps; f.h_j = (float)d.h_j; f.h_q = (float)d.h_q; f.h_nu = (float)d.h_nu;
     f.cs2_2tm = (float)d.cs2_2tm;
-    f.a_e = (float)d.a_e; f.g_u = (float)d.g_u; f.g_f = (float)d.g_f; f.a_j = (float)d.a_j; f.b_j = (float)d.b_j;
-    f.a_q = (float)d.a_q; f.b_q = (float)d.b_q; f.a_nu = (float)d.a_nu; f.b7 = (float)d.b7; f.b8 = (float)d.b8;
     f.tauT = (float)d.tauT; f.wg_den = (float)d.wg_den; f.gbeta = (float)d.gbeta; f.T0 = (float)d.T0;
     f.az = (float)d.az; f.lin_coef = (float)d.lin_coef; f.nl_coef = (float)d.nl_coef;
     f.T_hot = (float)d.T_hot; f.T_cold = (float)d.T_cold;
@@ -1773,7 +1695,6 @@ int lbm_destroy(lbm_handle* h) {
     return LBM_OK;
 }
 
-static TwoPlan two_plan(const lbm_params& p, int sms);
 static int launch_init(lbm_handle* h, const float* ur, const float* uz, const float* T) {
     if (int rc = wait_phi(h)) return rc;
     dim3 g = grid2d(h, 128);
@@ -1838,9 +1759,13 @@ int lbm_create(const lbm_params* p, lbm_handle** out) {
     ALLOC(h->result, 8 * sizeof(double));
     ALLOC(h->bad, sizeof(unsigned int));
 #undef ALLOC
-    // the two-step kernel serves FP32 storage in two buffers indexed with 32 bits; the discrete
-    // heater's wall reads a second row inward, which it does not carry
-    if (p->storage == LBM_F32 && !h->aa && !h->cf.heater && 14 * h->plane < ((int64_t)1 << 31)) h->two = two_plan(h->p, h->sms);
+    // several steps per launch: FP32 storage in two buffers indexed with 32 bits; the discrete
+    // heater's wall reads a second row inward, which those kernels do not carry
+    if (p->storage == LBM_F32 && !h->aa && !h->cf.heater && 14 * h->plane < ((int64_t)1 << 31)) {
+        h->c32 = consts32(h->cd, h->cf);
+        e = plan32(h->p, h->sms, &h->plan);
+        if (e != cudaSuccess) { lbm_destroy(h); return fail(LBM_ERR_CUDA, "plan32: %s", cudaGetErrorString(e)); }
+    }
     // uniform porosity eps_mean, then the cold start
     const int thr = 256;
     const unsigned blocks = (unsigned)((h->N + thr - 1) / thr);
@@ -2101,31 +2026,8 @@ static int launch_step(lbm_handle* h) {
     return LBM_OK;
 }
 
-// Rows per march of k_two.  A march of r rows takes r + 2 first and r second steps, so long
-// marches waste least, short ones fill the device: the r with the least (r + 2.5) x waves of
-// resident warps, half a wave added for the last one where there is more than one.  (4096 x
-// 8192, FP32: r = 32, 0.340 ms per step; 64 rows 0.355, 16 rows 0.343.)  The pipe's axis row
-// belongs to marches of the boundary form, so those take two rows there at least.
-static TwoPlan two_plan(const lbm_params& p, int sms) {
-    TwoPlan w, best;
-    w.first = (p.geometry == LBM_ANNULUS || p.geometry == LBM_ANNULUS_PERIODIC_Z) ? 1 : 0;
-    w.last = p.nr - 2;
-    w.strips = ((periodic_z(p.geometry) ? p.nz : p.nz & ~1) + TWO_COLS - 1) / TWO_COLS;
-    const double slots = (double)sms * LBM_TWO_MIN_BLOCKS * (BULK_THREADS / 32);
-    double cost = INFINITY;
-    for (int r = 1; r <= 256; ++r) {
-        w.rows = r;
-        w.erows = std::max(r * 5 / 8, w.first ? 1 : 2);
-        const double waves = (w.n_wall() + w.n_bulk()) / slots;
-        const double t = (r + 2.5) * (waves <= 1 ? 1.0 : waves + 0.5);
-        if (t < cost) { cost = t; best = w; }
-        if (r > w.last - w.first) break;
-    }
-    return best;
-}
-
-// Two steps in one pass.
-static int launch_two(lbm_handle* h) {
+// n steps in one launch (lbm_f32.h), boundary nodes included.
+static int launch_steps(lbm_handle* h, int n) {
     if (int rc = wait_phi(h)) return rc;
     cudaEvent_t e[4] = {nullptr, nullptr, nullptr, nullptr};   // bulk start / end; no wall kernel
     if (h->timing) {
@@ -2133,22 +2035,18 @@ static int launch_two(lbm_handle* h) {
         CK(cudaEventCreate(&e[1]));
         CK(cudaEventRecord(e[0], h->stream));
     }
-    const TwoPlan& w = h->two;
-    constexpr int WARPS = BULK_THREADS / 32;
-    const unsigned blocks = (unsigned)((w.n_wall() + WARPS - 1) / WARPS + (w.n_bulk() + WARPS - 1) / WARPS);
-    const auto A = bufp<LBM_F32>(h, h->cur), B = bufp<LBM_F32>(h, h->cur ^ 1);
-    if (h->p.nz & 1)
-        k_two<false><<<blocks, BULK_THREADS, 0, h->stream>>>(h->cf, A, B, (const float*)h->phi, (int)h->plane, w);
-    else
-        k_two<true><<<blocks, BULK_THREADS, 0, h->stream>>>(h->cf, A, B, (const float*)h->phi, (int)h->plane, w);
-    CK(cudaGetLastError());
+    const auto state = [&](int which) {
+        const Buf<LBM_F32> b = bufp<LBM_F32>(h, which);
+        return State32{b.f, b.g};
+    };
+    CK(launch32(h->plan, h->c32, state(h->cur), state(h->cur ^ 1), (const float*)h->phi, (int)h->plane, n, h->stream));
     if (h->timing) {
         CK(cudaEventRecord(e[1], h->stream));
         for (auto x : e) h->ev.push_back(x);
     }
     h->cur ^= 1;
-    h->info.steps += 2;
-    h->since_rebase += 2;
+    h->info.steps += n;
+    h->since_rebase += n;
     return LBM_OK;
 }
 
@@ -2157,12 +2055,10 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
     if (nsteps < 0) return fail(LBM_ERR_INVALID, "nsteps < 0");
     CK(cudaSetDevice(h->device));
     for (int64_t s = 0; s < nsteps;) {
-        // the last step is always a single one: it leaves the previous state in the other
-        // buffer (lbm_residual compares the two)
-        const bool two = h->two.strips && nsteps - s >= 3;
-        int rc = two ? launch_two(h) : launch_step(h);
+        const int n = h->plan.two.strips ? steps32(h->plan, nsteps - s) : 1;
+        const int rc = h->plan.two.strips ? launch_steps(h, n) : launch_step(h);
         if (rc) return rc;
-        s += two ? 2 : 1;
+        s += n;
     }
     return LBM_OK;
 }
@@ -2512,7 +2408,7 @@ int lbm_kernel_times(lbm_handle* h, double* bulk_ms, int64_t* bulk_launches, dou
         CK(cudaEventElapsedTime(&a, h->ev[i], h->ev[i + 1]));
         tb += a;
         nb += 1;
-        if (!h->ev[i + 2]) continue;   // a pass of two steps holds its boundary nodes
+        if (!h->ev[i + 2]) continue;   // a launch of several steps holds its boundary nodes
         CK(cudaEventElapsedTime(&b, h->ev[i + 2], h->ev[i + 3]));
         tw += b;
         nw += 1;
@@ -2932,6 +2828,12 @@ struct lbm_batch {
     int spin = STAGE_SPIN;            // try_wait rounds of its per-row waits
     int stage = 1;                    // 16-bit: staged tiles for the even-nz instances (lbm_batch_set_staging)
     int sms = 0;                      // multiprocessors of the device
+    // one launch per step (lbm_f32.h), where it serves every instance
+    bool step32 = false;
+    Inst32* d_inst32 = nullptr;
+    int2* d_blocks32 = nullptr;       // of the active instances: even nz, then odd nz
+    int nblocks32[2] = {0, 0};
+    size_t cap_blocks32 = 0;
     cudaGraphExec_t graph = nullptr;
     int64_t graph_steps = 0;
     int graph_parity = 0;             // batch parity the graph was captured at
@@ -2995,6 +2897,21 @@ static int batch_rebuild(lbm_batch* b) {
     }
     if (!st.empty())
         CK(cudaMemcpyAsync(b->d_stiles, st.data(), st.size() * sizeof(int4), cudaMemcpyHostToDevice, b->stream));
+    StepBlocks sb;
+    if (b->step32) {
+        sb = blocks32(b->p, act);
+        b->nblocks32[0] = (int)sb.even.size();
+        b->nblocks32[1] = (int)sb.odd.size();
+        sb.even.insert(sb.even.end(), sb.odd.begin(), sb.odd.end());
+        if (sb.even.size() > b->cap_blocks32) {
+            cudaFree(b->d_blocks32);
+            b->d_blocks32 = nullptr;
+            CK(cudaMalloc((void**)&b->d_blocks32, sb.even.size() * sizeof(int2)));
+            b->cap_blocks32 = sb.even.size();
+        }
+        if (!sb.even.empty())
+            CK(cudaMemcpyAsync(b->d_blocks32, sb.even.data(), sb.even.size() * sizeof(int2), cudaMemcpyHostToDevice, b->stream));
+    }
     b->ntiles = (int)tiles.size();
     b->nactive = (int)act.size();
     b->nwall = prefix.back();
@@ -3040,6 +2957,15 @@ static int batch_launch_step(lbm_batch* b) {
     // 16-bit storage: the refresh of lbm_step, every LBM_FREF_EVERY steps since the last
     if (b->storage != LBM_F32 && b->since_rebase >= LBM_FREF_EVERY)
         if (int rc = batch_launch_rebase_flow(b)) return rc;
+    if (b->step32) {
+        for (int odd = 0; odd < 2; ++odd)
+            if (b->nblocks32[odd])
+                CK(launch_batch32(b->d_inst32, b->d_blocks32 + (odd ? b->nblocks32[0] : 0), b->nblocks32[odd], odd != 0,
+                                  b->parity, b->stream));
+        b->parity ^= 1;
+        b->since_rebase += 1;
+        return LBM_OK;
+    }
     // the wall kernel reads only the pre-step states and writes only boundary nodes, which
     // the bulk kernels do not touch: it runs beside them on the wall stream
     CK(cudaEventRecord(b->wfork, b->stream));
@@ -3092,6 +3018,8 @@ int lbm_batch_destroy(lbm_batch* b) {
     cudaFree(b->fstage);
     cudaFree(b->d_tiles);
     cudaFree(b->d_stiles);
+    cudaFree(b->d_inst32);
+    cudaFree(b->d_blocks32);
     cudaFree(b->wait_status);
     cudaFree(b->d_active);
     cudaFree(b->d_prefix);
@@ -3170,6 +3098,22 @@ int lbm_batch_create(const lbm_params* p, int32_t n, lbm_batch** out) {
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(b->storage == LBM_F16 ? k_batch_stage<LBM_F16> : k_batch_stage<LBM_BF16>,
                                      cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+    }
+    b->step32 = true;
+    for (int i = 0; i < n; ++i) b->step32 = b->step32 && serves32(p[i]);
+    if (e == cudaSuccess && b->step32) {
+        std::vector<Inst32> inst(n);
+        for (int i = 0; i < n; ++i) {
+            inst[i].c = consts32(b->cd[i], b->desc[i].c);
+            for (int k = 0; k < 2; ++k) {
+                const Buf<LBM_F32> s = batch_buf<LBM_F32>(b, i, k);
+                inst[i].s[k] = State32{s.f, s.g};
+            }
+            inst[i].phi = (const float*)(b->pool + b->desc[i].off_phi);
+            inst[i].plane = (int)b->desc[i].plane;
+        }
+        e = cudaMalloc((void**)&b->d_inst32, n * sizeof(Inst32));
+        if (e == cudaSuccess) e = cudaMemcpy(b->d_inst32, inst.data(), n * sizeof(Inst32), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_desc, b->desc.data(), n * sizeof(InstDesc), cudaMemcpyHostToDevice,
                                               b->stream);

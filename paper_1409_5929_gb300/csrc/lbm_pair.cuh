@@ -86,7 +86,6 @@ struct RowC {
     float kT;      // tau_T / r
     float cs2r;    // c_s^2 / r
     float c2r;     // c_s^2 2 (tau - 1/2) / r
-    float c2rr;    // c_s^2 2 (tau - 1/2) / r^2
 };
 
 __device__ __forceinline__ RowC row_consts(const Consts<float>& c, int kr) {
@@ -100,7 +99,6 @@ __device__ __forceinline__ RowC row_consts(const Consts<float>& c, int kr) {
     q.kT = c.tauT * q.inv_r;
     q.cs2r = cs2<float>() * q.inv_r;
     q.c2r = c.cs2_2tm * q.inv_r;
-    q.c2rr = q.c2r * q.inv_r;
     return q;
 }
 

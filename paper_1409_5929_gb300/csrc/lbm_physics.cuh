@@ -45,9 +45,6 @@ struct Consts {
     R s_e, s_eps, s_j, s_q, s_nu;   // Eq. 23 with the rates of Sec. 4
     R h_e, h_eps, h_j, h_q, h_nu;   // 1 - s / 2 of each (the source weights of Eq. 21)
     R cs2_2tm;                      // c_s^2 2 (tau - 1/2)
-    // the same in the combinations of collide_two (lbm_two.cuh): s_e / 36, s_e / 12 and h_e / 6 (s_eps = s_e),
-    // s_j / 6 and h_j / 6, s_q / 12 and h_q / 12, s_nu / 4, h_nu / 2 and h_nu / 4
-    R a_e, g_u, g_f, a_j, b_j, a_q, b_q, a_nu, b7, b8;
     R tauT, wg_den;    // tau_T and 1 / (tau_T + 1/2)
     R gbeta, T0, az;   // buoyancy, reference temperature, external acceleration (z)
     R lin_coef;        // nu / K = lin_coef (mode 1) or lin_coef (1 - phi)^2 / phi^3 (mode 2)

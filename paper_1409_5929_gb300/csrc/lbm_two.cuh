@@ -26,10 +26,23 @@
 // size of the format's own error), while the time it won was 12 % (0.41 against 0.46 ms per
 // step, 4096 x 8192, FP16).
 #pragma once
+#include "lbm_f32.h"
 #include "lbm_pair.cuh"
 
 namespace lbm {
 
+// Row constants (RowC) and c_s^2 2 (tau - 1/2) / r^2.
+struct Row32 : RowC {
+    float c2rr;
+};
+__device__ __forceinline__ Row32 row_consts32(const Consts32& c, int kr) {
+    Row32 q;
+    static_cast<RowC&>(q) = row_consts(c, kr);
+    q.c2rr = q.c2r * q.inv_r;
+    return q;
+}
+
+constexpr int TWO_THREADS = 128;
 constexpr int TWO_COLS = 60;   // columns a strip stores (64 loaded)
 constexpr int TWO_KEEP = 17;   // 16-byte slots (two pairs) a thread keeps from row to row
 constexpr unsigned FULL = 0xffffffffu;
@@ -41,9 +54,7 @@ constexpr unsigned FULL = 0xffffffffu;
 struct Both { float v; };
 __device__ __forceinline__ Both both(float v) { return {v}; }
 __device__ __forceinline__ V2 operator+(V2 a, Both b) { return v2(__fadd_rn(a.v.x, b.v), __fadd_rn(a.v.y, b.v)); }
-__device__ __forceinline__ V2 operator+(Both a, V2 b) { return b + a; }
 __device__ __forceinline__ V2 operator*(V2 a, Both b) { return v2(__fmul_rn(a.v.x, b.v), __fmul_rn(a.v.y, b.v)); }
-__device__ __forceinline__ V2 operator*(Both a, V2 b) { return b * a; }
 __device__ __forceinline__ V2 fma2(V2 a, Both b, V2 c) {
     return v2(__fmaf_rn(a.v.x, b.v, c.v.x), __fmaf_rn(a.v.y, b.v, c.v.y));
 }
@@ -53,23 +64,41 @@ __device__ __forceinline__ V2 fma2(V2 a, V2 b, Both c) {
 __device__ __forceinline__ V2 fma2(V2 a, Both b, Both c) {
     return v2(__fmaf_rn(a.v.x, b.v, c.v), __fmaf_rn(a.v.y, b.v, c.v));
 }
+// The arithmetic below is written once for a pair (V = V2) and for a single node (V = float).
+__device__ __forceinline__ float operator+(float a, Both b) { return __fadd_rn(a, b.v); }
+__device__ __forceinline__ float operator*(float a, Both b) { return __fmul_rn(a, b.v); }
+__device__ __forceinline__ float fma2(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float fma2(float a, Both b, float c) { return __fmaf_rn(a, b.v, c); }
+__device__ __forceinline__ float fma2(float a, float b, Both c) { return __fmaf_rn(a, b, c.v); }
+__device__ __forceinline__ float fma2(float a, Both b, Both c) { return __fmaf_rn(a, b.v, c.v); }
+__device__ __forceinline__ V2 rcp_few(V2 x) { return rcp_fast(x); }       // reciprocal, square root: hardware
+__device__ __forceinline__ float rcp_few(float x) { return rcp_approx(x); }   // approximations
+__device__ __forceinline__ V2 sqrt_few(V2 x) { return sqrt_fast(x); }
+__device__ __forceinline__ float sqrt_few(float x) { return sqrt_approx(x); }
+template <class V> __device__ __forceinline__ V rcp_newton(V x) {   // and one Newton step (rcp_acc)
+    const V y = rcp_few(x);
+    return fma2(y, fma2(-x, y, both(1.0f)), y);
+}
+template <class V> __device__ __forceinline__ V all(float x);
+template <> __device__ __forceinline__ V2 all<V2>(float x) { return v2(x); }
+template <> __device__ __forceinline__ float all<float>(float x) { return x; }
 
 // Sums and differences of a pair's populations, shared by the recovery and the collision
 // (both are written on them; a packed multiply-add takes two issue cycles of the FMA pipe, the
 // pipe that bounds this code, so operations are what is saved: about 175 per pair and step
 // against 265 with the moments of Eq. 18 formed one by one).
-struct Sums {
-    V2 a, b;        // f_1 + .. + f_4, f_5 + .. + f_8
-    V2 s7, s8;      // m_7 = (f_1 + f_3) - (f_2 + f_4), m_8 = (f_5 + f_7) - (f_6 + f_8)
-    V2 d13, d24;    // f_1 - f_3, f_2 - f_4
-    V2 jr, jz;      // m_3, m_5
-    V2 m0;
+template <class V> struct Sums {
+    V a, b;         // f_1 + .. + f_4, f_5 + .. + f_8
+    V s7, s8;       // m_7 = (f_1 + f_3) - (f_2 + f_4), m_8 = (f_5 + f_7) - (f_6 + f_8)
+    V d13, d24;     // f_1 - f_3, f_2 - f_4
+    V jr, jz;       // m_3, m_5
+    V m0;
 };
 
-__device__ __forceinline__ Sums sums2(const V2* fh) {
-    Sums s;
-    const V2 s13 = fh[1] + fh[3], s24 = fh[2] + fh[4], s57 = fh[5] + fh[7], s68 = fh[6] + fh[8];
-    const V2 x57 = fh[5] - fh[7], x68 = fh[6] - fh[8];
+template <class V> __device__ __forceinline__ Sums<V> sums2(const V* fh) {
+    Sums<V> s;
+    const V s13 = fh[1] + fh[3], s24 = fh[2] + fh[4], s57 = fh[5] + fh[7], s68 = fh[6] + fh[8];
+    const V x57 = fh[5] - fh[7], x68 = fh[6] - fh[8];
     s.a = s13 + s24;
     s.b = s57 + s68;
     s.s7 = s13 - s24;
@@ -83,43 +112,45 @@ __device__ __forceinline__ Sums sums2(const V2* fh) {
 }
 
 // Eq. 8 per node (porous() of lbm_physics.cuh) for two nodes.
-__device__ __forceinline__ void porous_two(const Consts<float>& c, V2 phi, V2& lin, V2& nl, V2& inv_phi) {
-    const V2 ph2 = phi * phi;
-    const V2 ip3 = rcp_fast(ph2 * phi);
+template <class V>
+__device__ __forceinline__ void porous_two(const Consts32& c, V phi, V& lin, V& nl, V& inv_phi) {
+    const V ph2 = phi * phi;
+    const V ip3 = rcp_few(ph2 * phi);
     inv_phi = ph2 * ip3;
     if (c.porous_mode == 2) {
-        const V2 om = fma2(phi, both(-1.0f), both(1.0f));
+        const V om = fma2(phi, both(-1.0f), both(1.0f));
         lin = (om * om) * both(c.lin_coef) * ip3;
-        nl = c.ergun ? om * both(c.nl_coef) * ip3 : om * both(c.nl_coef) * sqrt_fast(ip3);
+        nl = c.ergun ? om * both(c.nl_coef) * ip3 : om * both(c.nl_coef) * sqrt_few(ip3);
     } else if (c.porous_mode == 1) {
-        lin = v2(c.lin_coef);
-        nl = c.ergun ? sqrt_fast(ip3) * both(c.nl_coef) : v2(c.nl_coef);
+        lin = all<V>(c.lin_coef);
+        nl = c.ergun ? sqrt_few(ip3) * both(c.nl_coef) : all<V>(c.nl_coef);
     } else {
-        lin = v2(0.f);
-        nl = v2(0.f);
+        lin = all<V>(0.f);
+        nl = all<V>(0.f);
     }
 }
 
 // recover() of lbm_physics.cuh (Eq. 26-30, 38) for two nodes; dT is relative to each
 // node's reference temperature T0 + R(x), rref = R(x).
-__device__ __forceinline__ void recover_two(const Consts<float>& c, const RowC& q, V2 phi, V2 lin, V2 nl,
-                                            const Sums& s, const V2* gh, V2 rref, V2& rho, V2& ur, V2& uz, V2& dT) {
+template <class V>
+__device__ __forceinline__ void recover_two(const Consts32& c, const Row32& q, V phi, V lin, V nl,
+                                            const Sums<V>& s, const V* gh, V rref, V& rho, V& ur, V& uz, V& dT) {
     dT = ((gh[0] + gh[1]) + (gh[2] + gh[3])) + gh[4];
     rho = fma2(s.m0, both(q.inv_r), both(1.0f));
-    const V2 Gz = fma2(dT + rref, both(c.gbeta), both(c.az));
-    const V2 inv_rho = rcp_acc(rho);
-    const V2 vr = fma2(s.m0, both(q.c1), s.jr) * inv_rho;
-    const V2 hp = phi * both(q.hr);
-    const V2 vz = fma2(s.jz, inv_rho, hp * Gz);
-    const V2 hd = phi * both(q.qr) * lin;
-    const V2 lr0 = hd + both(q.L0r);
-    const V2 lz0 = hd + both(q.hr);
+    const V Gz = fma2(dT + rref, both(c.gbeta), both(c.az));
+    const V inv_rho = rcp_newton(rho);
+    const V vr = fma2(s.m0, both(q.c1), s.jr) * inv_rho;
+    const V hp = phi * both(q.hr);
+    const V vz = fma2(s.jz, inv_rho, hp * Gz);
+    const V hd = phi * both(q.qr) * lin;
+    const V lr0 = hd + both(q.L0r);
+    const V lz0 = hd + both(q.hr);
     // Eq. 28 as in recover(), without a branch: x = 0 (no Forchheimer drag) adds 0
-    const V2 x = hp * nl * sqrt_fast(fma2(vr, vr, vz * vz));
-    const V2 Dr = fma2(x, rcp_fast(lr0 + sqrt_fast(fma2(lr0, lr0, x))), lr0 + lr0);
-    const V2 Dz = fma2(x, rcp_fast(lz0 + sqrt_fast(fma2(lz0, lz0, x))), lz0 + lz0);
-    ur = vr * rcp_acc(Dr);
-    uz = vz * rcp_acc(Dz);
+    const V x = hp * nl * sqrt_few(fma2(vr, vr, vz * vz));
+    const V Dr = fma2(x, rcp_few(lr0 + sqrt_few(fma2(lr0, lr0, x))), lr0 + lr0);
+    const V Dz = fma2(x, rcp_few(lz0 + sqrt_few(fma2(lz0, lz0, x))), lz0 + lz0);
+    ur = vr * rcp_newton(Dr);
+    uz = vz * rcp_newton(Dz);
 }
 
 // collide() of lbm_physics.cuh (Eq. 6, 21-25, 33-37) for two nodes, in place; rref = R(x).
@@ -132,39 +163,40 @@ __device__ __forceinline__ void recover_two(const Consts<float>& c, const RowC& 
 //   m_4 = m_3 - 3 (f_1 - f_3), m_6 = m_5 - 3 (f_2 - f_4).
 // As in collide(), Eq. 22 is applied to the change only, and mass and momentum of the change
 // are sums of exact multiples of its four parts.
-__device__ __forceinline__ void collide_two(const Consts<float>& c, const RowC& q, V2 phi, V2 lin, V2 nl, V2 inv_phi,
-                                            const Sums& s, V2* fh, V2* gh, V2 rref, V2 rho, V2 ur, V2 uz, V2 dT) {
-    const V2 Tb = rref + both(c.T0);   // the nodes' reference temperatures
-    const V2 T = Tb + dT;
-    const V2 uz2 = uz * uz;
-    const V2 u2 = fma2(ur, ur, uz2), ud = fma2(ur, ur, -uz2);
-    const V2 Gz = fma2(dT + rref, both(c.gbeta), both(c.az));
-    const V2 pd = phi * fma2(nl, sqrt_fast(u2), lin);
-    const V2 kr = pd + both(q.c2rr);
-    const V2 Ftr = fma2(-kr, ur, both(q.cs2r));   // Eq. 25
-    const V2 Ftz = fma2(-pd, uz, phi * Gz);
-    const V2 rr = rho * both(q.r);
-    const V2 rri = rr * inv_phi;
-    const V2 e3 = rr * ur, e5 = rr * uz;
+template <class V>
+__device__ __forceinline__ void collide_two(const Consts32& c, const Row32& q, V phi, V lin, V nl, V inv_phi,
+                                            const Sums<V>& s, V* fh, V* gh, V rref, V rho, V ur, V uz, V dT) {
+    const V Tb = rref + both(c.T0);   // the nodes' reference temperatures
+    const V T = Tb + dT;
+    const V uz2 = uz * uz;
+    const V u2 = fma2(ur, ur, uz2), ud = fma2(ur, ur, -uz2);
+    const V Gz = fma2(dT + rref, both(c.gbeta), both(c.az));
+    const V pd = phi * fma2(nl, sqrt_few(u2), lin);
+    const V kr = pd + both(q.c2rr);
+    const V Ftr = fma2(-kr, ur, both(q.cs2r));   // Eq. 25
+    const V Ftz = fma2(-pd, uz, phi * Gz);
+    const V rr = rho * both(q.r);
+    const V rri = rr * inv_phi;
+    const V e3 = rr * ur, e5 = rr * uz;
     // S_3 without its rest constant c_s^2 (see collide()), S_5
-    const V2 S3 = fma2(-kr, e3, s.m0 * both(q.cs2r));
-    const V2 S5 = rr * Ftz;
-    const V2 uzFz = uz * Ftz;
-    const V2 pq = fma2(ur, Ftr, uzFz), pm = fma2(ur, Ftr, -uzFz);
-    const V2 G = rri * fma2(u2, both(c.g_u), pq * both(c.g_f));
-    const V2 A1 = fma2(fma2(fh[0], both(-2.0f), fma2(s.b, both(4.0f), s.a)), both(-c.a_e), G);
-    const V2 A2 = fma2(fh[0] - s.a, both(-c.g_u), -G);
-    const V2 b14 = fma2(A2, both(-2.0f), -A1), b58 = fma2(A1, both(2.0f), A2);
-    const V2 a7 = fma2(s.s7, both(-c.a_nu), rri * fma2(ud, both(c.a_nu), pm * both(c.b7)));
-    const V2 a8 = fma2(s.s8, both(-c.a_nu), rri * fma2(ur * uz, both(c.a_nu), fma2(ur, Ftz, uz * Ftr) * both(c.b8)));
-    const V2 a3 = fma2(s.jr - e3, both(-c.a_j), S3 * both(c.b_j));
-    const V2 a4 = fma2(fma2(s.d13, both(-3.0f), s.jr + e3), both(-c.a_q), S3 * both(-c.b_q));
-    const V2 a5 = fma2(s.jz - e5, both(-c.a_j), S5 * both(c.b_j));
-    const V2 a6 = fma2(fma2(s.d24, both(-3.0f), s.jz + e5), both(-c.a_q), S5 * both(-c.b_q));
-    const V2 x3 = fma2(a4, both(-2.0f), a3), x5 = fma2(a6, both(-2.0f), a5);
-    const V2 y3 = a3 + a4, y5 = a5 + a6;
-    const V2 yp = y3 + y5, ym = y3 - y5;
-    const V2 bp = b14 + a7, bm = b14 - a7, cp = b58 + a8, cm = b58 - a8;
+    const V S3 = fma2(-kr, e3, s.m0 * both(q.cs2r));
+    const V S5 = rr * Ftz;
+    const V uzFz = uz * Ftz;
+    const V pq = fma2(ur, Ftr, uzFz), pm = fma2(ur, Ftr, -uzFz);
+    const V G = rri * fma2(u2, both(c.g_u), pq * both(c.g_f));
+    const V A1 = fma2(fma2(fh[0], both(-2.0f), fma2(s.b, both(4.0f), s.a)), both(-c.a_e), G);
+    const V A2 = fma2(fh[0] - s.a, both(-c.g_u), -G);
+    const V b14 = fma2(A2, both(-2.0f), -A1), b58 = fma2(A1, both(2.0f), A2);
+    const V a7 = fma2(s.s7, both(-c.a_nu), rri * fma2(ud, both(c.a_nu), pm * both(c.b7)));
+    const V a8 = fma2(s.s8, both(-c.a_nu), rri * fma2(ur * uz, both(c.a_nu), fma2(ur, Ftz, uz * Ftr) * both(c.b8)));
+    const V a3 = fma2(s.jr - e3, both(-c.a_j), S3 * both(c.b_j));
+    const V a4 = fma2(fma2(s.d13, both(-3.0f), s.jr + e3), both(-c.a_q), S3 * both(-c.b_q));
+    const V a5 = fma2(s.jz - e5, both(-c.a_j), S5 * both(c.b_j));
+    const V a6 = fma2(fma2(s.d24, both(-3.0f), s.jz + e5), both(-c.a_q), S5 * both(-c.b_q));
+    const V x3 = fma2(a4, both(-2.0f), a3), x5 = fma2(a6, both(-2.0f), a5);
+    const V y3 = a3 + a4, y5 = a5 + a6;
+    const V yp = y3 + y5, ym = y3 - y5;
+    const V bp = b14 + a7, bm = b14 - a7, cp = b58 + a8, cm = b58 - a8;
     fh[0] = fma2(A2 - A1, both(4.0f), fh[0]);
     fh[1] += bp + x3;
     fh[2] += bm + x5;
@@ -176,14 +208,14 @@ __device__ __forceinline__ void collide_two(const Consts<float>& c, const RowC& 
     fh[8] += cm + ym;
     // D2Q5 (Eq. 33, 35-37), relative to T0 + R(x)
     const float wd = c.wg_den, wp = (1.0f + q.kT) * wd, wm = (1.0f - q.kT) * wd;
-    const V2 cu = ur * both(-q.inv_r);
-    const V2 hT = T * both(0.5f);
-    const V2 Tr = hT * ur, Tz = hT * uz;
-    const V2 t1 = dT * both(0.1f);
-    const V2 g1e = t1 + Tr, g3e = t1 - Tr;
-    const V2 g2e = t1 + Tz, g4e = t1 - Tz;
-    const V2 g0e = fma2(t1, both(-4.0f), dT);
-    const V2 wT0 = Tb * both(0.6f), wT1 = Tb * both(0.1f);
+    const V cu = ur * both(-q.inv_r);
+    const V hT = T * both(0.5f);
+    const V Tr = hT * ur, Tz = hT * uz;
+    const V t1 = dT * both(0.1f);
+    const V g1e = t1 + Tr, g3e = t1 - Tr;
+    const V g2e = t1 + Tz, g4e = t1 - Tz;
+    const V g0e = fma2(t1, both(-4.0f), dT);
+    const V wT0 = Tb * both(0.6f), wT1 = Tb * both(0.1f);
     gh[0] = fma2(cu, g0e + wT0, fma2(gh[0] - g0e, both(-wd), gh[0]));
     gh[1] = fma2(cu, g1e + wT1, fma2(gh[1] - g1e, both(-wp), gh[1]));
     gh[2] = fma2(cu, g2e + wT1, fma2(gh[2] - g2e, both(-wd), gh[2]));
@@ -195,27 +227,15 @@ __device__ __forceinline__ void collide_two(const Consts<float>& c, const RowC& 
 __device__ __forceinline__ V2 from_left(V2 x) { return v2(__shfl_up_sync(FULL, x.v.y, 1), x.v.x); }
 __device__ __forceinline__ V2 from_right(V2 x) { return v2(x.v.y, __shfl_down_sync(FULL, x.v.x, 1)); }
 
-// Boundary rebuild (rebuild_flow, rebuild_thermal of lbm_physics.cuh) of the boundary lanes of
-// row j from the pulled state of row p (p = j except on wall rows): fh, gh, m0, rho, ur, uz, dT
-// hold that state with its reference reff and 1/phi iphf, and receive the boundary state on
-// the boundary lanes.  phj, refj: porosity and temperature reference of row j.
-template <bool ODD>
-__device__ __forceinline__ void wall_pair(const Consts<float>& c, int p, int j, int ca, V2 (&fh)[9], V2 (&gh)[5],
-                                          V2 m0, V2& rho, V2& ur, V2& uz, V2& dT, V2 iphf, V2 reff, V2 phj, V2 refj) {
-    const int nz = c.nz, cb = ca + 1;
-    const bool closed = !c.periodic;
-    const int k0 = node_class(c.geometry, c.nr, nz, j, ca), k1 = node_class(c.geometry, c.nr, nz, j, cb);
-    // (periodic z: only wall rows come here, and the columns past the ends are wrapped ones)
-    const bool w0 = (!closed || (ca >= 0 && ca < nz)) && is_wall(k0);
-    const bool w1 = (!closed || (cb >= 0 && cb < nz)) && is_wall(k1);
-    const bool l_first = closed && ca == 0, h_last = closed && cb == nz - 1;
-    const bool l_last = ODD && closed && ca == nz - 1;
-    // the neighbour's value on each lane
-    const auto nb = [&](V2 x) {
-        float up = 0.f;
-        if (ODD) up = __shfl_up_sync(FULL, x.v.y, 1);
-        return v2(l_first ? x.v.y : (l_last ? up : x.v.x), h_last ? x.v.x : x.v.y);
-    };
+// Boundary rebuild (rebuild_flow, rebuild_thermal of lbm_physics.cuh) of the boundary lanes
+// (w0, w1; classes k0, k1) of row j from the pulled state of row p (p = j except on wall rows):
+// fh, gh, m0, rho, ur, uz, dT hold that state with its reference reff and 1/phi iphf, and receive
+// the boundary state on the boundary lanes.  nb(x): the interior neighbours' values, lane by
+// lane.  phj, refj: porosity and temperature reference of row j.
+template <class NB>
+__device__ __forceinline__ void wall_rebuild(const Consts32& c, int p, int j, int k0, int k1, bool w0, bool w1,
+                                             const NB& nb, V2 (&fh)[9], V2 (&gh)[5], V2 m0, V2& rho, V2& ur, V2& uz,
+                                             V2& dT, V2 iphf, V2 reff, V2 phj, V2 refj) {
     const auto put = [&](V2& x, V2 w) { x = v2(w0 ? w.v.x : x.v.x, w1 ? w.v.y : x.v.y); };
     const float rf = c.r0 + float(p), rb = c.r0 + float(j);
     const float inv_rf = rcp_acc(rf), inv_rb = rcp_acc(rb);
@@ -274,6 +294,40 @@ __device__ __forceinline__ void wall_pair(const Consts<float>& c, int p, int j, 
     put(dT, dTb);
 }
 
+// The same where the neighbour of an end column sits in the other lane of the pair or (ODD: odd
+// nz) in the previous thread; ca: the pair's first column.
+template <bool ODD>
+__device__ __forceinline__ void wall_pair(const Consts32& c, int p, int j, int ca, V2 (&fh)[9], V2 (&gh)[5],
+                                          V2 m0, V2& rho, V2& ur, V2& uz, V2& dT, V2 iphf, V2 reff, V2 phj, V2 refj) {
+    const int nz = c.nz, cb = ca + 1;
+    const bool closed = !c.periodic;
+    const int k0 = node_class(c.geometry, c.nr, nz, j, ca), k1 = node_class(c.geometry, c.nr, nz, j, cb);
+    // (periodic z: only wall rows come here, and the columns past the ends are wrapped ones)
+    const bool w0 = (!closed || (ca >= 0 && ca < nz)) && is_wall(k0);
+    const bool w1 = (!closed || (cb >= 0 && cb < nz)) && is_wall(k1);
+    const bool l_first = closed && ca == 0, h_last = closed && cb == nz - 1;
+    const bool l_last = ODD && closed && ca == nz - 1;
+    const auto nb = [&](V2 x) {
+        float up = 0.f;
+        if (ODD) up = __shfl_up_sync(FULL, x.v.y, 1);
+        return v2(l_first ? x.v.y : (l_last ? up : x.v.x), h_last ? x.v.x : x.v.y);
+    };
+    wall_rebuild(c, p, j, k0, k1, w0, w1, nb, fh, gh, m0, rho, ur, uz, dT, iphf, reff, phj, refj);
+}
+
+// Two columns of a plane (VEC: aligned neighbours), and the stores of both or the first.
+template <bool VEC> __device__ __forceinline__ V2 ld_two(const float* p, int la, int lb) {
+    if (VEC) return {__ldg(reinterpret_cast<const float2*>(p + la))};
+    return v2(__ldg(p + la), __ldg(p + lb));
+}
+template <bool VEC> __device__ __forceinline__ void st_two(float* p, V2 v, bool second) {
+    if (VEC) {
+        *reinterpret_cast<float2*>(p) = v.v;
+    } else {
+        p[0] = v.v.x;
+        if (second) p[1] = v.v.y;
+    }
+}
 // Two columns of the reference plane R(x), as loaded and as floats.
 template <bool VEC> __device__ __forceinline__ uint32_t ld_ref(const __half* p, int la, int lb) {
     if (VEC) return __ldg(reinterpret_cast<const uint32_t*>(p + la));
@@ -287,7 +341,7 @@ __device__ __forceinline__ V2 ref_of(uint32_t w) { return {__half22float2(*reint
 // strip before: two_plan); wall >= 0: ka = kb is the neighbour row of wall row `wall`, and that wall
 // row is written instead.  VEC: nz even.  WALLS: the march meets boundary nodes.
 template <bool VEC, bool WALLS>
-__device__ __forceinline__ void two_march(const Consts<float>& c, const Buf<LBM_F32>& A, const Buf<LBM_F32>& B,
+__device__ __forceinline__ void two_march(const Consts32& c, const State32& A, const State32& B,
                                           const float* __restrict__ phi, int plane, int s, int ka, int kb, int wall,
                                           float4* __restrict__ ring) {
     const int nr = c.nr, nz = c.nz, lane = threadIdx.x & 31;
@@ -316,10 +370,10 @@ __device__ __forceinline__ void two_march(const Consts<float>& c, const Buf<LBM_
     // reference (row j again in the half of its parity)
     float4* const keep = ring + threadIdx.x;
     const auto put = [&](int slot, V2 a, V2 b) {
-        keep[slot * BULK_THREADS] = make_float4(a.v.x, a.v.y, b.v.x, b.v.y);
+        keep[slot * TWO_THREADS] = make_float4(a.v.x, a.v.y, b.v.x, b.v.y);
     };
     const auto take = [&](int slot, V2& a, V2& b) {
-        const float4 t = keep[slot * BULK_THREADS];
+        const float4 t = keep[slot * TWO_THREADS];
         a = v2(t.x, t.y);
         b = v2(t.z, t.w);
     };
@@ -354,7 +408,7 @@ __device__ __forceinline__ void two_march(const Consts<float>& c, const Buf<LBM_
             const bool axis = WALLS && p == 0;   // pipe axis: the e_r = +1 sources are row 0's mirror image
             const int row = p * nz, rowp = row + nz, rowm = axis ? row : row - nz;
             const int i1 = axis ? 3 : 1, i5 = axis ? 6 : 5, i8 = axis ? 7 : 8;
-            const auto ld = [&](const float* q) { return ld2(q, la, lb, VEC); };
+            const auto ld = [&](const float* q) { return ld_two<VEC>(q, la, lb); };
             fh[0] = ld(F + row);
             fh[1] = ld(F + (i1 * plane + rowm));
             fh[2] = ld(F + (2 * plane + row));
@@ -382,7 +436,7 @@ __device__ __forceinline__ void two_march(const Consts<float>& c, const Buf<LBM_
             put(u + 1, t3, t4);
             put(u + 2, ph, lin);
             put(u + 3, nl, iph);
-            reinterpret_cast<uint32_t&>(keep[(u + 4) * BULK_THREADS]) = wo;
+            reinterpret_cast<uint32_t&>(keep[(u + 4) * TWO_THREADS]) = wo;
             gh[1] += t1;
             gh[3] += t3;
             fh[2] = from_left(fh[2]);
@@ -394,19 +448,19 @@ __device__ __forceinline__ void two_march(const Consts<float>& c, const Buf<LBM_
             gh[2] = from_left(gh[2]) + t2;
             gh[4] = from_right(gh[4]) + t4;
             V2 rho, ur, uz, dT;
-            Sums sm = sums2(fh);
-            recover_two(c, row_consts(c, p), ph, lin, nl, sm, gh, R, rho, ur, uz, dT);
+            Sums<V2> sm = sums2(fh);
+            recover_two(c, row_consts32(c, p), ph, lin, nl, sm, gh, R, rho, ur, uz, dT);
             if (WALLS && (edge || p != j)) {
                 const V2 Rf = R, iphf = iph;
                 if (p != j) {
-                    ph = ld2(phi + j * nz, la, lb, VEC);
+                    ph = ld_two<VEC>(phi + j * nz, la, lb);
                     R = ref_of(ld_ref<VEC>(c.tref + j * nz, la, lb));
                     porous_two(c, ph, lin, nl, iph);
                 }
                 wall_pair<!VEC>(c, p, j, ca, fh, gh, sm.m0, rho, ur, uz, dT, iphf, Rf, ph, R);
                 sm = sums2(fh);
             }
-            collide_two(c, row_consts(c, j), ph, lin, nl, iph, sm, fh, gh, R, rho, ur, uz, dT);
+            collide_two(c, row_consts32(c, j), ph, lin, nl, iph, sm, fh, gh, R, rho, ur, uz, dT);
             fh[2] = from_left(fh[2]);
             fh[5] = from_left(fh[5]);
             fh[6] = from_left(fh[6]);
@@ -439,32 +493,32 @@ __device__ __forceinline__ void two_march(const Consts<float>& c, const Buf<LBM_
             take(u + 1, t3, t4);
             take(u + 2, ph, lin);
             take(u + 3, nl, iph);
-            V2 R = ref_of(reinterpret_cast<const uint32_t&>(keep[(u + 4) * BULK_THREADS]));
+            V2 R = ref_of(reinterpret_cast<const uint32_t&>(keep[(u + 4) * TWO_THREADS]));
             g[1] += t1;
             g[2] += t2;
             g[3] += t3;
             g[4] += t4;
             V2 rho, ur, uz, dT;
-            Sums sm = sums2(f);
-            recover_two(c, row_consts(c, k), ph, lin, nl, sm, g, R, rho, ur, uz, dT);
+            Sums<V2> sm = sums2(f);
+            recover_two(c, row_consts32(c, k), ph, lin, nl, sm, g, R, rho, ur, uz, dT);
             if (WALLS && (edge || o != k)) {
                 const V2 Rf = R, iphf = iph;
                 if (o != k) {
-                    ph = ld2(phi + o * nz, la, lb, VEC);
+                    ph = ld_two<VEC>(phi + o * nz, la, lb);
                     R = ref_of(ld_ref<VEC>(c.tref + o * nz, la, lb));
                     porous_two(c, ph, lin, nl, iph);
                 }
                 wall_pair<!VEC>(c, k, o, ca, f, g, sm.m0, rho, ur, uz, dT, iphf, Rf, ph, R);
                 sm = sums2(f);
             }
-            collide_two(c, row_consts(c, o), ph, lin, nl, iph, sm, f, g, R, rho, ur, uz, dT);
+            collide_two(c, row_consts32(c, o), ph, lin, nl, iph, sm, f, g, R, rho, ur, uz, dT);
             float* __restrict__ Fo = B.f + o * nz;
             float* __restrict__ Go = B.g + o * nz;
             if (st0) {
 #pragma unroll
-                for (int i = 0; i < 9; ++i) st2(Fo + i * plane, ca, f[i], true, VEC || st1, VEC);
+                for (int i = 0; i < 9; ++i) st_two<VEC>(Fo + i * plane + ca, f[i], st1);
 #pragma unroll
-                for (int i = 0; i < 5; ++i) st2(Go + i * plane, ca, g[i], true, VEC || st1, VEC);
+                for (int i = 0; i < 5; ++i) st_two<VEC>(Go + i * plane + ca, g[i], st1);
             }
         }
     }
