@@ -291,7 +291,8 @@ int lbm_export_populations(lbm_handle *h, int32_t row0, int32_t nrows, double *f
 int lbm_get_info(lbm_handle *h, lbm_info *out);
 
 /* Bounded waits of the staged 16-bit bulk kernel (not an operation of the paper).  With
- * 16-bit storage, even nz and grids of at least 16 blocks per SM, the bulk step copies
+ * 16-bit storage, even nz and large grids (more than eight million nodes; at least 16 blocks
+ * per SM once a limit was set here), the bulk step copies
  * each row's source segments into shared memory with bulk copies whose completion every
  * thread awaits for at most `rounds` polls (default a few seconds).
  * A wait that runs out marks the handle: the block drains its copies in flight and
@@ -390,7 +391,8 @@ int lbm_batch_pipe_nusselt(lbm_batch *b, int32_t i, double *nu, int32_t nz);
  * step count in lbm_batch_get_info includes them). */
 int lbm_batch_tune(lbm_batch *b, int32_t steps, int32_t *cols, int32_t *rows, float *ms_per_step);
 /* lbm_set_wait_limit and lbm_wait_status for the batch's staged 16-bit bulk kernel
- * (instances with even nz; the tuned tile shape then serves the odd-nz instances and the
+ * (instances with even nz of batches of more than five million nodes, or of any batch once a
+ * limit was set; the tuned tile shape then serves the odd-nz instances and the
  * reference refresh).  lbm_batch_run checks the status after every check interval. */
 int lbm_batch_set_wait_limit(lbm_batch *b, int rounds);
 int lbm_batch_wait_status(lbm_batch *b, int clear);

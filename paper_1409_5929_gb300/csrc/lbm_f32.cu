@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "lbm_dependent.h"
 #include "lbm_step32.cuh"
 #include "lbm_tile.cuh"
 #include "lbm_two.cuh"
@@ -114,24 +115,6 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile(const Consts32 c, cons
                                                           int plane, const TilePlan w, int steps) {
     extern __shared__ float tile_sm[];
     tile_steps(c, A, B, phi, plane, w, steps, tile_sm);
-}
-
-// Launch with programmatic dependent launch: the kernel's blocks may start while the launch before
-// it still runs and wait for its end (griddepcontrol.wait) before their first access to memory.
-template <class K, class... Args>
-static cudaError_t launch_dependent(K kernel, unsigned blocks, unsigned threads, size_t shared, cudaStream_t stream,
-                                    Args... args) {
-    cudaLaunchAttribute at = {};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = shared;
-    cfg.stream = stream;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // Rows per march of k_two.  A march of r rows takes r + 2 first and r second steps, so long

@@ -1,4 +1,5 @@
-"""GPU tests of the launches that take several steps (FP32 storage): lbm_step(n) takes up to ten
+"""GPU tests of the launches that hold their boundary nodes, and of those that take several steps
+(FP32 storage): lbm_step(n) takes up to ten
 steps per launch on small grids (tiles with a halo) and pairs of steps on larger ones (strips of
 60 columns and chunks of rows), boundary nodes included; lbm_step(1) takes single ones.  The same
 problem advanced both ways, at the sizes where that can go wrong: grids smaller than a tile, a
@@ -96,5 +97,54 @@ def test_batch_passes_match_single_steps(lbm):
     for i in range(len(shapes)):
         for x, y in zip(a.moments(i), b.moments(i)):
             assert _err(x, y) <= 1e-5, (shapes[i], _err(x, y))
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("storage", ["f16", "bf16"])
+@pytest.mark.parametrize("geometry,nr,nz", [(0, 1086, 2104), (0, 1086, 2102), (1, 1086, 2102), (2, 1086, 2104),
+                                            (0, 700, 1301), (1, 60, 121), (2, 61, 97), (3, 41, 181), (0, 3, 3), (0, 4, 5)])
+def test_16bit_launch_with_boundary_nodes(lbm, storage, geometry, nr, nz):
+    """16-bit storage: the launch that holds its boundary nodes (even nz, odd nz with its shifted
+    pairs, periodic odd nz, the smallest grids) against in-place storage in the codec's error
+    against FP32, and, on grids that can take it, against the staged kernel, which setting a wait
+    limit selects: the same update on the same values, a flipped 16-bit rounding apart
+    (test_gpu_stage's bound)."""
+    n = 60
+    ref, a, b = (_solver(lbm, geometry, nr, nz, sto, inplace=k) for sto, k in (("f32", 0), (storage, 0), (storage, 1)))
+    for s in (ref, a, b):
+        s.step(n)
+    m = [s.moments() for s in (ref, a, b)]
+    u = [np.stack(x[1:3]) for x in m]
+    assert _err(u[1], u[0]) <= 1.5 * _err(u[2], u[0]) + 1e-5
+    assert _err(m[1][3], m[0][3]) <= 1.5 * _err(m[2][3], m[0][3]) + 1e-5
+    if nr > 1000:
+        c = _solver(lbm, geometry, nr, nz, storage)
+        lbm.lbm_set_wait_limit(c.h, (1 << 22) + 1)
+        c.step(n)
+        assert lbm.lbm_wait_status(c.h) == lbm.LBM_OK
+        assert max(float(np.abs(np.asarray(x, np.float64) - y).max()) for x, y in zip(c.moments(), m[1])) <= 2e-5
+        c.close()
+    for s in (ref, a, b):
+        s.close()
+
+
+@pytest.mark.parametrize("storage", ["f16", "bf16"])
+def test_16bit_batch_launch_matches_staged(lbm, storage):
+    """The same for the batch: one launch per step from global loads against the staged tiles that a
+    wait limit selects, every geometry, odd and even nz."""
+    shapes = [(0, 40, 262), (0, 37, 121), (1, 21, 520), (2, 25, 130), (3, 41, 180), (0, 3, 3)]
+    kw = {0: dict(Ra=1e5, Da=1e-3, Pr=0.71), 1: dict(Ra=1e4, Da=5e-3, body_accel_z=2e-6),
+          2: dict(Ra=0.0, tau_nu=0.8, Da=0.05, F_eps=0.0, body_accel_z=2e-6),
+          3: dict(Ra=0.0, Da=1e-2, eps_mean=1.0, F_eps=0.0, Pr=0.7, tau_nu=0.62, u_in=0.05)}
+    p = [lbm.lbm_params_default(nr=nr, nz=nz, geometry=g, storage=storage, init_noise=0.02, **kw[g]) for g, nr, nz in shapes]
+    a, b = lbm.Batch(p), lbm.Batch(p)
+    lbm.lbm_batch_set_wait_limit(b.b, (1 << 22) + 1)
+    for x in (a, b):
+        x.step(61)
+        x.run(20, 10, -1.0)
+    assert lbm.lbm_batch_wait_status(b.b) == lbm.LBM_OK
+    for i in range(len(shapes)):
+        assert max(float(np.abs(np.asarray(x, np.float64) - y).max()) for x, y in zip(a.moments(i), b.moments(i))) <= 2e-5
     a.close()
     b.close()
