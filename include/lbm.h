@@ -391,7 +391,7 @@ int lbm_batch_pipe_nusselt(lbm_batch *b, int32_t i, double *nu, int32_t nz);
  * step count in lbm_batch_get_info includes them). */
 int lbm_batch_tune(lbm_batch *b, int32_t steps, int32_t *cols, int32_t *rows, float *ms_per_step);
 /* lbm_set_wait_limit and lbm_wait_status for the batch's staged 16-bit bulk kernel
- * (instances with even nz of batches of more than five million nodes, or of any batch once a
+ * (instances with even nz of batches of more than eight million nodes, or of any batch once a
  * limit was set; the tuned tile shape then serves the odd-nz instances and the
  * reference refresh).  lbm_batch_run checks the status after every check interval. */
 int lbm_batch_set_wait_limit(lbm_batch *b, int rounds);

@@ -2173,7 +2173,7 @@ static int batch_stage_rows(const lbm_batch* b, const std::vector<int>& act) {
 // 16-bit batches up to this many nodes take one launch per step from global loads (lbm_16.h), larger
 // ones the staged tiles with the wall kernel beside them.  A batch whose wait limit was set runs
 // staged: its waits are what the limit is for.
-constexpr int64_t BATCH_STEP16_NODES = 5000000;
+constexpr int64_t BATCH_STEP16_NODES = 8000000;
 static int batch_rebuild(lbm_batch* b) {
     std::vector<int4> tiles, odd;   // tiles of instances with odd nz last (k_batch_bulk's VEC)
     std::vector<int> act, prefix(1, 0);

@@ -102,12 +102,12 @@ __global__ void __launch_bounds__(BULK_THREADS, 6) k_step16(const Step16 s, int 
 }
 
 // The same for the instances of a batch, whose constants are read from shared memory.  16 instances
-// of 64 to 160 rows (450 k nodes, FP16): 10.0 us per step (19.0 with staged tiles and the forked wall
-// kernel); 16 of 200 to 400 (3.6 M nodes, BF16) 70 against 76; 64 of 64 to 512 (12.2 M nodes) 242
+// of 64 to 160 rows (450 k nodes, FP16): 10.2 us per step (19.0 with staged tiles and the forked wall
+// kernel); 16 of 200 to 400 (3.6 M nodes, BF16) 68 against 76; 64 of 64 to 512 (12.2 M nodes) 232
 // against 231, where the staged tiles serve.  The staged tiles with the boundary nodes in their
-// launch: 234.
+// launch: 234.  Six blocks per SM; with five 70 and 242, with seven 72 and 245.
 template <int STO, bool VEC>
-__global__ void __launch_bounds__(BULK_THREADS, 5) k_batch_step16(const Step16* __restrict__ inst,
+__global__ void __launch_bounds__(BULK_THREADS, 6) k_batch_step16(const Step16* __restrict__ inst,
                                                                   const int2* __restrict__ blocks, int from) {
     __shared__ Step16 s;
     const int2 b = blocks[blockIdx.x];   // the lists and constants are not written by a launch
