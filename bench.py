@@ -47,15 +47,15 @@ TRAFFIC = {("f32", 4096, 8192): ("e47fb4700593f444", 2089953280 + 1827634944),
 
 
 def _kernel_hash() -> str:
-    """Hash of the bulk kernels' own source: csrc/lbm_physics.cuh, csrc/lbm_pair.cuh and
-    csrc/lbm.cu up to the end of the bulk kernels (where k_wall begins); host code and
-    other kernels further down do not change the traffic record's validity."""
+    """Hash of the bulk kernels' own source: the headers they are built from, csrc/lbm_f32.cu, and
+    csrc/lbm.cu up to the end of the bulk kernels (where k_wall begins); host code and other
+    kernels further down do not change the traffic record's validity."""
     import hashlib
 
     d = os.path.join(ROOT, "paper_1409_5929_gb300", "csrc")
     h = hashlib.sha256()
-    h.update(open(os.path.join(d, "lbm_physics.cuh"), "rb").read())
-    h.update(open(os.path.join(d, "lbm_pair.cuh"), "rb").read())
+    for name in ("lbm_physics.cuh", "lbm_pair.cuh", "lbm_nodes.cuh", "lbm_two.cuh", "lbm_f32.cu"):
+        h.update(open(os.path.join(d, name), "rb").read())
     src = open(os.path.join(d, "lbm.cu"), "rb").read()
     k = src.find(b"__global__ void k_wall(")
     cut = src.rfind(b"template <", 0, k) if k > 0 else -1

@@ -14,15 +14,16 @@
 //   fref:             nr*nz flow references Q(x), 4 x FP16 each (16-bit storage).
 //   macro snapshots, reduction scratch, staging: only for diagnostics.
 //
-// A step is two launches on the handle's stream:
-//   k_bulk  every non-wall node: pull (Eq. 22, 33), recovery (Eq. 26-30, 38),
-//           collision (Eq. 21-24, 33-37), store.  Grid (nz / 128, nr).  With
-//           16-bit storage k_bulk_stage: two z-adjacent nodes per thread on the
-//           packed FP32 instructions (lbm_pair.cuh).
-//   k_wall  every wall node: rebuild from the interior neighbour by
-//           non-equilibrium extrapolation (Sec. 4, ref. [47]), collision with
-//           u = 0 and the wall temperature, store.  One thread per wall node.
-// Both read only the source buffer and write disjoint nodes of the destination.
+// A step in two buffers is one launch that holds its boundary nodes (FP32: lbm_f32.cu, on small and
+// large grids several steps per launch; 16-bit storage: lbm_16.cu), except
+//   k_bulk_stage + k_wall   16-bit storage on large grids: every non-wall node (pull, Eq. 22, 33;
+//           recovery, Eq. 26-30, 38; collision, Eq. 21-24, 33-37; store), row sources staged in
+//           shared memory; then every wall node (rebuild from the interior neighbour by
+//           non-equilibrium extrapolation, Sec. 4, ref. [47], collision with u = 0 and the
+//           wall temperature), one thread each;
+//   k_bulk + k_wall         one node per thread: in-place storage (the wall kernel first), the
+//           discrete heater, and grids beyond 32-bit indices.
+// Both kernels of a pair read only the source buffer and write disjoint nodes of the destination.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda.h>
@@ -1363,6 +1364,16 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
 
 static int launch_moments(lbm_handle* h, int which, float* rho, float* ur, float* uz, float* T) {
     if (int rc = wait_phi(h)) return rc;
+    if (h->plan.two.strips) {   // FP32 storage in two buffers (lbm_f32.h)
+        const Buf<LBM_F32> b = bufp<LBM_F32>(h, which);
+        CK(launch_fields32(h->c32, State32{b.f, b.g}, (const float*)h->phi, (int)h->plane, rho, ur, uz, T, h->stream));
+        return LBM_OK;
+    }
+    if (h->step16) {            // 16-bit storage in two buffers (lbm_16.h)
+        h->s16.phi = (const float*)h->phi;
+        CK(launch_fields16(h->p.storage, h->s16, which, rho, ur, uz, T, h->stream));
+        return LBM_OK;
+    }
     const dim3 g = grid2d(h, 128);
     DISPATCH_LAY(cur_lay(h), DISPATCH_STO(h->p.storage,
                  k_moments<S_, L_><<<g, 128, 0, h->stream>>>(h->cf, bufp<S_>(h, which), (const PP<S_>*)h->phi,
@@ -2127,6 +2138,8 @@ struct lbm_batch {
     int stage = 1;                    // 16-bit: staged tiles for the even-nz instances (lbm_batch_set_staging)
     int sms = 0;                      // multiprocessors of the device
     // one launch per step (lbm_16.h)
+    std::vector<Step16> inst16;
+    std::vector<Inst32> inst32;
     Step16* d_inst16 = nullptr;
     int2* d_blocks16 = nullptr;       // of the active instances: even nz, then odd nz
     int nblocks16[2] = {0, 0};
@@ -2435,7 +2448,8 @@ int lbm_batch_create(const lbm_params* p, int32_t n, lbm_batch** out) {
                                      cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
     }
     if (e == cudaSuccess && b->storage != LBM_F32) {
-        std::vector<Step16> inst(n);
+        std::vector<Step16>& inst = b->inst16;
+        inst.resize(n);
         for (int i = 0; i < n; ++i) {
             const InstDesc& d = b->desc[i];
             inst[i].c = d.c;
@@ -2452,7 +2466,8 @@ int lbm_batch_create(const lbm_params* p, int32_t n, lbm_batch** out) {
     b->step32 = true;
     for (int i = 0; i < n; ++i) b->step32 = b->step32 && serves32(p[i]);
     if (e == cudaSuccess && b->step32) {
-        std::vector<Inst32> inst(n);
+        std::vector<Inst32>& inst = b->inst32;
+        inst.resize(n);
         for (int i = 0; i < n; ++i) {
             inst[i].c = consts32(b->cd[i], b->desc[i].c);
             for (int k = 0; k < 2; ++k) {
@@ -2629,7 +2644,9 @@ int lbm_batch_run(lbm_batch* b, int64_t max_steps, int64_t check_every, double t
     while (total < max_steps && b->nactive > 0) {
         const int64_t k = std::min(check_every, max_steps - total);
         // reference refresh before every check interval, as lbm_run does
-        if (b->storage == LBM_F32) {
+        if (b->step32) {
+            CK(launch_batch_rebase32(b->d_inst32, b->d_active, b->nactive, b->parity, b->stream));
+        } else if (b->storage == LBM_F32) {
             for (int i = 0; i < b->n; ++i)
                 if (b->active[i] && (rc = batch_rebase_one(b, i))) return rc;
         } else if ((rc = batch_launch_rebase_flow(b))) {
@@ -2769,10 +2786,17 @@ int lbm_batch_moments(lbm_batch* b, int32_t i, float* rho, float* ur, float* uz,
     float* outs[4] = {rho, ur, uz, T};
     float* dst[4];
     for (int j = 0; j < 4; ++j) dst[j] = on_device ? outs[j] : (outs[j] ? m + j * d.plane : nullptr);
-    DISPATCH_STO(b->storage, k_moments<S_><<<g, 128, 0, b->stream>>>(d.c, batch_buf<S_>(b, i, b->cur_parity(i)),
-                                                                      (const PP<S_>*)(b->pool + d.off_phi), d.plane,
-                                                                      dst[0], dst[1], dst[2], dst[3]));
-    CK(cudaGetLastError());
+    const int cur = b->cur_parity(i);
+    if (b->storage != LBM_F32) {
+        CK(launch_fields16(b->storage, b->inst16[i], cur, dst[0], dst[1], dst[2], dst[3], b->stream));
+    } else if (b->step32) {
+        CK(launch_fields32(b->inst32[i].c, b->inst32[i].s[cur], b->inst32[i].phi, b->inst32[i].plane, dst[0], dst[1], dst[2],
+                           dst[3], b->stream));
+    } else {
+        k_moments<LBM_F32><<<g, 128, 0, b->stream>>>(d.c, batch_buf<LBM_F32>(b, i, cur), (const float*)(b->pool + d.off_phi),
+                                                     d.plane, dst[0], dst[1], dst[2], dst[3]);
+        CK(cudaGetLastError());
+    }
     if (!on_device)
         for (int j = 0; j < 4; ++j)
             if (outs[j]) CK(cudaMemcpyAsync(outs[j], dst[j], N * sizeof(float), cudaMemcpyDeviceToHost, b->stream));

@@ -101,6 +101,75 @@ __global__ void __launch_bounds__(BULK_THREADS, 6) k_step16(const Step16 s, int 
     }
 }
 
+// Fields of interior pair n: update_pair's pull and recovery.
+template <int STO, bool VEC>
+__device__ __forceinline__ void fields_pair16(const Consts<float>& c, const Buf<STO>& A, const float* __restrict__ phi,
+                                              int plane, int n, const Fields& o) {
+    const int nz = c.nz, P = (nz + 1) >> 1, y = n / P, kr = step_row0(c.geometry) + y, kz = 2 * (n - y * P);
+    const bool pz = c.periodic != 0, in1 = kz + 1 < nz;
+    const bool st0 = pz || (kz > 0 && kz < nz - 1), st1 = in1 && (pz || kz + 1 < nz - 1);
+    if (kr >= c.nr - 1 || (!st0 && !st1)) return;
+    const int zc = in1 ? kz + 1 : kz, zm = kz > 0 ? kz - 1 : (pz ? nz - 1 : 0), z0 = in1 ? kz + 1 : (pz ? 0 : nz - 1);
+    const int z1 = kz + 2 < nz ? kz + 2 : (pz ? kz + 2 - nz : nz - 1);
+    const int row = kr * nz, rowp = row + nz, rowm = kr == 0 ? row : row - nz;   // (pipe axis: mirror image)
+    const int p1 = kr == 0 ? 3 : 1, p5 = kr == 0 ? 6 : 5, p8 = kr == 0 ? 7 : 8;
+    const auto* __restrict__ F = A.f;
+    const float* __restrict__ G = A.g;
+    const auto own = [&](const auto* p, int r) { return ld2(p, r + kz, r + zc, VEC); };
+    const auto left = [&](const auto* p, int r) { return ld2(p, r + zm, r + kz, false); };
+    const auto right = [&](const auto* p, int r) { return ld2(p, r + z0, r + z1, false); };
+    V2 fh[9] = {own(F, row), own(F + p1 * plane, rowm), left(F + 2 * plane, row), own(F + 3 * plane, rowp),
+                right(F + 4 * plane, row), left(F + p5 * plane, rowm), left(F + 6 * plane, rowp),
+                right(F + 7 * plane, rowp), right(F + p8 * plane, rowm)};
+    V2 gh[5] = {own(G, row), own(G + p1 * plane, rowm), left(G + 2 * plane, row), own(G + 3 * plane, rowp),
+                right(G + 4 * plane, row)};
+    const V2 ph = own(phi, row);
+    const Q2 q0 = ldq2(c.fref, row + kz, row + zc, VEC);
+    const V2 R = q0.R;
+    const auto add = [&](int r, int a, int b, bool vec, int i0, int s0, int i1, int s1, int i2, int s2) {
+        const Q2 q = ldq2(c.fref, r + a, r + b, vec);
+        if (i0 >= 0) fh[i0] += fref_delta2(s0, q);
+        if (i1 >= 0) fh[i1] += fref_delta2(s1, q);
+        if (i2 >= 0) gh[i2] += 0.1f * (q.R - R);
+    };
+    fh[0] += fref_delta2(0, q0);
+    add(row, zm, kz, false, 2, 2, -1, 0, 2, 0);
+    add(row, z0, z1, false, 4, 4, -1, 0, 4, 0);
+    add(rowm, kz, zc, VEC, 1, p1, -1, 0, 1, 0);
+    add(rowm, zm, kz, false, 5, p5, -1, 0, -1, 0);
+    add(rowm, z0, z1, false, 8, p8, -1, 0, -1, 0);
+    add(rowp, kz, zc, VEC, 3, 3, -1, 0, 3, 0);
+    add(rowp, zm, kz, false, 6, 6, -1, 0, -1, 0);
+    add(rowp, z0, z1, false, 7, 7, -1, 0, -1, 0);
+    V2 lin, nl, iph, m0, rho, ur, uz, dT;
+    porous2(c, ph, lin, nl, iph);
+    recover2(c, row_consts(c, kr), ph, lin, nl, fh, gh, R, m0, rho, ur, uz, dT);
+    put_pair(o, row + kz, st0, st1, rho, ur, uz, (c.T0 + R) + dT);
+}
+template <int STO, bool VEC>
+__global__ void __launch_bounds__(BULK_THREADS, 8) k_fields16(const Step16 s, int which, int walls, const Fields o) {
+    const int wall_blocks = (walls + BULK_THREADS - 1) / BULK_THREADS;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const Buf<STO> A = buf16<STO>(s, which);
+    if ((int)blockIdx.x < wall_blocks) {
+        const int n = blockIdx.x * BULK_THREADS + threadIdx.x;
+        if (n >= walls) return;
+        const Consts<float>& c = s.c;
+        int kr, kz;
+        wall_node(c.geometry, c.nr, c.nz, n, kr, kz);
+        float fh[9], gh[5], m0, rho, ur, uz, dT, ref;
+        wall_state<STO, float>(c, A, s.phi, s.plane, node_class(c.geometry, c.nr, c.nz, kr, kz), kr, kz, fh, gh, m0, rho, ur,
+                               uz, dT, ref);
+        const float v[4] = {rho, ur, uz, (c.T0 + ref) + dT};
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (o.p[k]) o.p[k][kr * c.nz + kz] = v[k];
+    } else {
+        fields_pair16<STO, VEC>(s.c, A, s.phi, (int)s.plane, ((int)blockIdx.x - wall_blocks) * BULK_THREADS + threadIdx.x, o);
+    }
+}
+
 // The same for the instances of a batch, whose constants are read from shared memory.  16 instances
 // of 64 to 160 rows (450 k nodes, FP16): 10.2 us per step (19.0 with staged tiles and the forked wall
 // kernel); 16 of 200 to 400 (3.6 M nodes, BF16) 68 against 76; 64 of 64 to 512 (12.2 M nodes) 232
@@ -153,6 +222,16 @@ cudaError_t launch_batch16(int storage, const Step16* inst, const int2* blocks, 
     const auto k = storage == LBM_F16 ? (odd_nz ? k_batch_step16<LBM_F16, false> : k_batch_step16<LBM_F16, true>)
                                       : (odd_nz ? k_batch_step16<LBM_BF16, false> : k_batch_step16<LBM_BF16, true>);
     return launch_dependent(k, (unsigned)n, BULK_THREADS, 0, stream, inst, blocks, from);
+}
+
+cudaError_t launch_fields16(int storage, const Step16& s, int which, float* rho, float* ur, float* uz, float* T,
+                            cudaStream_t stream) {
+    const Consts<float>& c = s.c;
+    const int walls = step_walls(c.geometry, c.nr, c.nz), pairs = step_pairs(c.geometry, c.nr, c.nz);
+    const unsigned blocks = (walls + BULK_THREADS - 1) / BULK_THREADS + (pairs + BULK_THREADS - 1) / BULK_THREADS;
+    const auto k = storage == LBM_F16 ? (c.nz & 1 ? k_fields16<LBM_F16, false> : k_fields16<LBM_F16, true>)
+                                      : (c.nz & 1 ? k_fields16<LBM_BF16, false> : k_fields16<LBM_BF16, true>);
+    return launch_dependent(k, blocks, BULK_THREADS, 0, stream, s, which, walls, fields_of(c.nz, rho, ur, uz, T));
 }
 
 }  // namespace lbm

@@ -23,7 +23,11 @@ struct Step16 {
 // One step of a problem from buffer `from` to the other, the interior from global loads.
 cudaError_t launch16(int storage, const Step16& s, int from, cudaStream_t stream);
 
-// The same for the instances of a batch.  Blocks: (2 instance + kind, first interior pair or boundary
+// Fields of the state in buffer `which`, as lbm_moments (outputs nr nz floats in device memory or NULL).
+cudaError_t launch_fields16(int storage, const Step16& s, int which, float* rho, float* ur, float* uz, float* T,
+                            cudaStream_t stream);
+
+// One step of the instances of a batch.  Blocks: (2 instance + kind, first interior pair or boundary
 // node), kind 1 for boundary nodes.
 struct Blocks16 {
     std::vector<int2> even, odd;   // instances with even and odd nz

@@ -68,6 +68,10 @@ int steps32(const Plan32& w, int64_t left);
 cudaError_t launch32(const Plan32& w, const Consts32& c, const State32& A, const State32& B, const float* phi, int plane,
                      int steps, cudaStream_t stream);
 
+// Fields of a state, as lbm_moments (outputs nr nz floats in device memory or NULL).
+cudaError_t launch_fields32(const Consts32& c, const State32& A, const float* phi, int plane, float* rho, float* ur,
+                            float* uz, float* T, cudaStream_t stream);
+
 // ---- batches: one launch per step for every active instance
 struct Inst32 {
     Consts32 c;
@@ -82,6 +86,8 @@ struct StepBlocks {
 };
 bool serves32(const lbm_params& p);   // FP32 storage, no discrete heater
 StepBlocks blocks32(const std::vector<lbm_params>& p, const std::vector<int>& act);
+// lbm_rebase of the instances act[0 .. n - 1] (device memory), state in buffer `which`.
+cudaError_t launch_batch_rebase32(const Inst32* inst, const int* act, int n, int which, cudaStream_t stream);
 cudaError_t launch_batch32(const Inst32* inst, const int2* blocks, int n, bool odd_nz, int parity, cudaStream_t stream);
 
 }  // namespace lbm
