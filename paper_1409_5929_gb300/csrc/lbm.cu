@@ -2245,8 +2245,6 @@ static int batch_rebuild(lbm_batch* b) {
         sb.even.insert(sb.even.end(), sb.odd.begin(), sb.odd.end());
         if (sb.even.size() > b->cap_blocks32) {
             cudaFree(b->d_blocks32);
-    cudaFree(b->d_inst16);
-    cudaFree(b->d_blocks16);
             b->d_blocks32 = nullptr;
             CK(cudaMalloc((void**)&b->d_blocks32, sb.even.size() * sizeof(int2)));
             b->cap_blocks32 = sb.even.size();

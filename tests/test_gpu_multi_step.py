@@ -73,9 +73,9 @@ def test_two_step_pass_matches_single_steps(lbm, geometry, nr, nz):
 
 
 def test_batch_passes_match_single_steps(lbm):
-    """The batch's two-step launches (marches of every instance in one list, even and odd nz,
-    every geometry, instances smaller than a strip) against single steps of the same batch, with
-    an odd tail and with captured intervals whose number of pairs is odd."""
+    """The batch's launches (the nodes of every instance in one list, even and odd nz,
+    every geometry, instances smaller than a block) against single steps of the same batch, with
+    an odd number of steps and with captured intervals."""
     shapes = [(0, 64, 128), (0, 37, 121), (1, 23, 120), (1, 5, 61), (2, 25, 130), (3, 41, 181), (0, 3, 3), (0, 160, 320)]
 
     def make():
