@@ -38,12 +38,12 @@ SAMPLE_NR, SAMPLE_NZ = 256, 512   # bounded CPU sample: the same recipe on a 256
 E2E_STEPS = 50                    # minimum length of the end-to-end window (steps)
 
 
-# DRAM traffic of one k_bulk launch on the 4096 x 8192 workload (dram__bytes_read.sum +
+# DRAM traffic of one bulk launch (FP32: k_two, two steps) on the 4096 x 8192 workload (dram__bytes_read.sum +
 # dram__bytes_write.sum of the bulk kernel in one single-pass ncu capture of this
 # benchmark), valid only for the bulk kernel's source it was taken on (_kernel_hash).
-TRAFFIC = {("f32", 4096, 8192): ("e47fb4700593f444", 2089953280 + 1827634944),
-           ("f16", 4096, 8192): ("e47fb4700593f444", 1690808064 + 1227835648),
-           ("bf16", 4096, 8192): ("e47fb4700593f444", 1689640704 + 1228074496)}
+TRAFFIC = {("f32", 4096, 8192): ("255f586a56e33446", 2285157632 + 1841550336),
+           ("f16", 4096, 8192): ("255f586a56e33446", 1690624768 + 1227723520),
+           ("bf16", 4096, 8192): ("255f586a56e33446", 1689783808 + 1227624448)}
 
 
 def _kernel_hash() -> str:
@@ -201,7 +201,7 @@ def _bulk_kernel(storage: str, inplace: int) -> str:
     two-column kernel for 16-bit storage on two buffers."""
     if inplace:
         return f"k_bulk<{storage}>"
-    return "k_two (k_bulk<f32> for the last steps)" if storage == "f32" else f"k_bulk_stage<{storage}>"
+    return "k_two (k_step for the last steps)" if storage == "f32" else f"k_bulk_stage<{storage}>"
 
 
 def storage_variant(lbm, storage, phi, steps, warmup, peak, inplace=0):
