@@ -24,9 +24,9 @@ __device__ __forceinline__ void wall16(const Consts<float>& c, const Buf<STO>& A
     wall_node(c.geometry, c.nr, c.nz, n, kr, kz);
     const int cls = node_class(c.geometry, c.nr, c.nz, kr, kz);
     float fh[9], gh[5], m0, rho, urb, uzb, dTb, refb;
-    wall_state<STO, float>(c, A, phi, plane, cls, kr, kz, fh, gh, m0, rho, urb, uzb, dTb, refb);
+    wall_state<STO, float, LAY_N, true>(c, A, phi, plane, cls, kr, kz, fh, gh, m0, rho, urb, uzb, dTb, refb);
     const int64_t m = (int64_t)kr * c.nz + kz;
-    const float r = c.r0 + float(kr), ph = ldv(phi + m);
+    const float r = c.r0 + float(kr), ph = ldv<true>(phi + m);
     float lin, nl, iph;
     porous(c, ph, lin, nl, iph);
     collide(c, r, rcp_acc(r), ph, lin, nl, iph, fh, gh, refb, m0, rho, urb, uzb, dTb);
@@ -46,8 +46,8 @@ __device__ __forceinline__ void pair_odd(const Consts<float>& c, const Buf<STO>&
     if (!st0 && !st1) return;
     const auto* __restrict__ F = A.f;
     const float* __restrict__ G = A.g;
-    const auto vec = [&](const auto* p, int o) { return ld2(p, o, o + 1, true); };
-    const auto two = [&](const auto* p, int o) { return ld2(p, o, o + 1, false); };
+    const auto vec = [&](const auto* p, int o) { return ld2<true>(p, o, o + 1, true); };
+    const auto two = [&](const auto* p, int o) { return ld2<true>(p, o, o + 1, false); };
     V2 fh[9], gh[5];
     fh[0] = vec(F, row + kz0);
     fh[1] = two(F + plane, rowm + kz0);
@@ -66,7 +66,7 @@ __device__ __forceinline__ void pair_odd(const Consts<float>& c, const Buf<STO>&
     const V2 ph = vec(phi, row + kz0);
     const auto qw = [&](int rs, int cs) {
         const int o = (rs == 0 ? rowm : rs == 1 ? row : rowp) + kz0 + cs - 1;
-        return ldq2(c.fref, o, o + 1, (rs == 1) == (cs == 1));
+        return ldq2<true>(c.fref, o, o + 1, (rs == 1) == (cs == 1));
     };
     pair_finish<STO, true>(c, B, plane, kr, row, kz0, 1, 5, 8, fh, gh, ph, qw, st0, st1);
 }
@@ -79,7 +79,7 @@ __device__ __forceinline__ void inner16(const Consts<float>& c, const Buf<STO>& 
     if (!VEC && !c.periodic && kr >= 2 && kr <= c.nr - 3) {
         pair_odd<STO>(c, A, B, phi, plane, kr, n - y * P);
     } else {
-        update_pair<STO, VEC>(c, A, B, phi, plane, kr, 1, 2 * (n - y * P));
+        update_pair<STO, VEC, true>(c, A, B, phi, plane, kr, 1, 2 * (n - y * P));
     }
 }
 
@@ -115,19 +115,19 @@ __device__ __forceinline__ void fields_pair16(const Consts<float>& c, const Buf<
     const int p1 = kr == 0 ? 3 : 1, p5 = kr == 0 ? 6 : 5, p8 = kr == 0 ? 7 : 8;
     const auto* __restrict__ F = A.f;
     const float* __restrict__ G = A.g;
-    const auto own = [&](const auto* p, int r) { return ld2(p, r + kz, r + zc, VEC); };
-    const auto left = [&](const auto* p, int r) { return ld2(p, r + zm, r + kz, false); };
-    const auto right = [&](const auto* p, int r) { return ld2(p, r + z0, r + z1, false); };
+    const auto own = [&](const auto* p, int r) { return ld2<true>(p, r + kz, r + zc, VEC); };
+    const auto left = [&](const auto* p, int r) { return ld2<true>(p, r + zm, r + kz, false); };
+    const auto right = [&](const auto* p, int r) { return ld2<true>(p, r + z0, r + z1, false); };
     V2 fh[9] = {own(F, row), own(F + p1 * plane, rowm), left(F + 2 * plane, row), own(F + 3 * plane, rowp),
                 right(F + 4 * plane, row), left(F + p5 * plane, rowm), left(F + 6 * plane, rowp),
                 right(F + 7 * plane, rowp), right(F + p8 * plane, rowm)};
     V2 gh[5] = {own(G, row), own(G + p1 * plane, rowm), left(G + 2 * plane, row), own(G + 3 * plane, rowp),
                 right(G + 4 * plane, row)};
     const V2 ph = own(phi, row);
-    const Q2 q0 = ldq2(c.fref, row + kz, row + zc, VEC);
+    const Q2 q0 = ldq2<true>(c.fref, row + kz, row + zc, VEC);
     const V2 R = q0.R;
     const auto add = [&](int r, int a, int b, bool vec, int i0, int s0, int i1, int s1, int i2, int s2) {
-        const Q2 q = ldq2(c.fref, r + a, r + b, vec);
+        const Q2 q = ldq2<true>(c.fref, r + a, r + b, vec);
         if (i0 >= 0) fh[i0] += fref_delta2(s0, q);
         if (i1 >= 0) fh[i1] += fref_delta2(s1, q);
         if (i2 >= 0) gh[i2] += 0.1f * (q.R - R);
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(BULK_THREADS, 8) k_fields16(const Step16 s, in
         int kr, kz;
         wall_node(c.geometry, c.nr, c.nz, n, kr, kz);
         float fh[9], gh[5], m0, rho, ur, uz, dT, ref;
-        wall_state<STO, float>(c, A, s.phi, s.plane, node_class(c.geometry, c.nr, c.nz, kr, kz), kr, kz, fh, gh, m0, rho, ur,
+        wall_state<STO, float, LAY_N, true>(c, A, s.phi, s.plane, node_class(c.geometry, c.nr, c.nz, kr, kz), kr, kz, fh, gh, m0, rho, ur,
                                uz, dT, ref);
         const float v[4] = {rho, ur, uz, (c.T0 + ref) + dT};
 #pragma unroll

@@ -26,7 +26,7 @@ using namespace lbm;
 template <bool VEC>
 __global__ void __launch_bounds__(TWO_THREADS, LBM_TWO_MIN_BLOCKS) k_two(const Consts32 c, const State32 A,
                                                                          const State32 B,
-                                                                         const float* __restrict__ phi, int plane,
+                                                                         const float* phi, int plane,
                                                                          const TwoPlan w) {
     __shared__ float4 ring[TWO_KEEP * TWO_THREADS];
     constexpr int WARPS = TWO_THREADS / 32;
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(TWO_THREADS, LBM_TWO_MIN_BLOCKS) k_two(const C
 template <bool VEC>
 __global__ void __launch_bounds__(STEP_THREADS, LBM_STEP_MIN_BLOCKS) k_step(const Consts32 c, const State32 A,
                                                                             const State32 B,
-                                                                            const float* __restrict__ phi, int plane,
+                                                                            const float* phi, int plane,
                                                                             int walls) {
     const int wall_blocks = (walls + STEP_THREADS - 1) / STEP_THREADS;
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_STEP_MIN_BLOCKS) k_step(cons
 // the boundary rebuild in the same warps): one step of 48 x 96 and its fields 8.2 -> 7.1 us,
 // 4096 x 8192 0.42 -> 0.36 ms (FP16 storage, k_fields16: 0.48 -> 0.36).
 template <bool VEC>
-__global__ void __launch_bounds__(STEP_THREADS, 8) k_fields(const Consts32 c, const State32 A, const float* __restrict__ phi,
+__global__ void __launch_bounds__(STEP_THREADS, 8) k_fields(const Consts32 c, const State32 A, const float* phi,
                                                             int plane, int walls, const Fields o) {
     const int wall_blocks = (walls + STEP_THREADS - 1) / STEP_THREADS;
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(256) k_batch_rebase(const Inst32* __restrict__
 // Several steps per launch on small grids (lbm_tile.cuh).  48 x 96: 1.5 us per step (10.3 as two
 // launches per step, 4.7 with k_two; 1.9 without the dependent launch); 100 x 200: 1.7 us.
 __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile(const Consts32 c, const State32 A,
-                                                          const State32 B, const float* __restrict__ phi,
+                                                          const State32 B, const float* phi,
                                                           int plane, const TilePlan w, int steps) {
     extern __shared__ float tile_sm[];
     tile_steps(c, A, B, phi, plane, w, steps, tile_sm);

@@ -18,9 +18,20 @@ using namespace lbm;
 // 16 bits the per-step change of g - wT T0, of order 0.05, falls below the format's
 // resolution and the temperature field stagnates); porosity always FP32 (in FP16 its
 // half-ulp, 2.4e-4 relative near 0.7, moves the Darcy drag of Eq. 8 by about 2e-3).
-__device__ __forceinline__ float ldv(const float* p) { return __ldg(p); }
-__device__ __forceinline__ float ldv(const __half* p) { return __half2float(__ldg(p)); }
-__device__ __forceinline__ float ldv(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
+//
+// Loads.  DEP: the kernel is launched dependently (lbm_dependent.h), so it is resident while the
+// launch before it may still write the state, the references or the porosity; only an ordinary load
+// stays behind its wait.  The read-only load (__ldg) wants data that no one writes during the whole
+// life of the kernel.
+template <bool DEP, class T> __device__ __forceinline__ T ld1(const T* p) {
+    if constexpr (DEP) return *p;
+    else return __ldg(p);
+}
+template <bool DEP = false> __device__ __forceinline__ float ldv(const float* p) { return ld1<DEP>(p); }
+template <bool DEP = false> __device__ __forceinline__ float ldv(const __half* p) { return __half2float(ld1<DEP>(p)); }
+template <bool DEP = false> __device__ __forceinline__ float ldv(const __nv_bfloat16* p) {
+    return __bfloat162float(ld1<DEP>(p));
+}
 __device__ __forceinline__ void stv(float* p, float v) { *p = v; }
 __device__ __forceinline__ void stv(__half* p, float v) { *p = __float2half_rn(v); }
 __device__ __forceinline__ void stv(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
@@ -127,7 +138,7 @@ template <int STO> __host__ __device__ constexpr bool has_fref() { return STO !=
 // plain copy of ft_i(x - e_i) (see lbm_physics.cuh), plus, with 16-bit storage, the
 // reference part D_pop(Q(source)) of the value the source node stored.  src receives the
 // source nodes (for the temperature reference).
-template <int STO, int LAY, typename R, typename I>
+template <int STO, int LAY, bool DEP, typename R, typename I>
 __device__ __forceinline__ void pull_raw(const Consts<R>& c, const Buf<STO>& A, I plane, int kr, int kz, R* fh,
                                          R* gh, I* src) {
     I loc[9];
@@ -137,12 +148,12 @@ __device__ __forceinline__ void pull_raw(const Consts<R>& c, const Buf<STO>& A, 
     const auto* __restrict__ G = A.g;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-        float v = ldv(F + lp[i] * plane + loc[i]);
+        float v = ldv<DEP>(F + lp[i] * plane + loc[i]);
         if constexpr (has_fref<STO>()) v += fref_delta(sp[i], fref_unpack(c.fref[src[i]]));
         fh[i] = R(v);
     }
 #pragma unroll
-    for (int i = 0; i < 5; ++i) gh[i] = R(ldv(G + lp[i] * plane + loc[i]));
+    for (int i = 0; i < 5; ++i) gh[i] = R(ldv<DEP>(G + lp[i] * plane + loc[i]));
 }
 
 // Re-reference pulled thermal deviations to the node's R(x): gh_i += wT_i (R(x - e_i) - R(x))
@@ -174,11 +185,11 @@ __device__ __forceinline__ float tref_at(const Consts<R>& c, I n) {
 
 // Pull (Eq. 22) from layout LAY with the thermal deviations re-referenced to R(x), which
 // *rref receives (on the pipe axis row g_1 comes from the node's own mirror image).
-template <int STO, typename R, typename I = int64_t, int LAY = LAY_N>
+template <int STO, typename R, typename I = int64_t, int LAY = LAY_N, bool DEP = false>
 __device__ __forceinline__ void pull(const Consts<R>& c, const Buf<STO>& A, I plane, int kr, int kz, R* fh, R* gh,
                                      R& rref) {
     I src[9];
-    pull_raw<STO, LAY, R, I>(c, A, plane, kr, kz, fh, gh, src);
+    pull_raw<STO, LAY, DEP, R, I>(c, A, plane, kr, kz, fh, gh, src);
     rref = R(tref_at<STO>(c, (I)kr * c.nz + kz));
     reref(gh, rref, R(tref_at<STO>(c, src[1])), R(tref_at<STO>(c, src[2])), R(tref_at<STO>(c, src[3])),
           R(tref_at<STO>(c, src[4])));
@@ -221,7 +232,7 @@ __device__ __forceinline__ void store(const Consts<float>& c, const Buf<STO>& B,
 // rho from Eq. 26.  Walls: u_b = 0, rho_b = rho_f, T_b = T_hot (inner), T_cold (outer),
 // T_f (adiabatic top and bottom).  Pipe inlet: u_b = (0, u_in), rho_b = rho_f, T_b = T_hot;
 // outlet: u_b = u_f, T_b = T_f, rho_b = 1 (zero gradient of u and T, density held).
-template <int STO, typename R, int LAY = LAY_N>
+template <int STO, typename R, int LAY = LAY_N, bool DEP = false>
 __device__ __forceinline__ void wall_state(const Consts<R>& c, const Buf<STO> A,
                                            const typename St<STO>::P* __restrict__ phi, int64_t plane, int cls,
                                            int kr, int kz, R* fh, R* gh, R& m0, R& rho, R& urb, R& uzb, R& dTb,
@@ -229,9 +240,9 @@ __device__ __forceinline__ void wall_state(const Consts<R>& c, const Buf<STO> A,
     int fr, fz;
     fluid_neighbour(c.geometry, c.nr, c.nz, cls, kr, kz, fr, fz);
     R fhf[9], ghf[5], reff;
-    pull<STO, R, int64_t, LAY>(c, A, plane, fr, fz, fhf, ghf, reff);
+    pull<STO, R, int64_t, LAY, DEP>(c, A, plane, fr, fz, fhf, ghf, reff);
     const R rf = c.r0 + R(fr), rb = c.r0 + R(kr);
-    const R phif = R(ldv(phi + (int64_t)fr * c.nz + fz));
+    const R phif = R(ldv<DEP>(phi + (int64_t)fr * c.nz + fz));
     R m0f, rhof, urf, uzf, dTf, lin, nl, ipf;
     porous(c, phif, lin, nl, ipf);
     recover(c, rf, rcp_acc(rf), phif, lin, nl, fhf, ghf, reff, m0f, rhof, urf, uzf, dTf);
@@ -247,7 +258,7 @@ __device__ __forceinline__ void wall_state(const Consts<R>& c, const Buf<STO> A,
         drhob = R(0);
         rhob = R(1);
     }
-    if (cls >= INLET) ipb = rcp_acc(R(ldv(phi + (int64_t)kr * c.nz + kz)));
+    if (cls >= INLET) ipb = rcp_acc(R(ldv<DEP>(phi + (int64_t)kr * c.nz + kz)));
     rebuild_flow(rb, rf, ipb, ipf, drhob, rhob, urb, uzb, m0f, rhof, urf, uzf, fhf, fh);
     // deviations relative to this boundary node's own reference R_b
     refb = R(tref_at<STO>(c, (int64_t)kr * c.nz + kz));
@@ -260,7 +271,7 @@ __device__ __forceinline__ void wall_state(const Consts<R>& c, const Buf<STO> A,
         // corners (diagonal neighbour) take T_f
         if (fz == kz) {
             R f2[9], g2[5], ref2;
-            pull<STO, R, int64_t, LAY>(c, A, plane, 2, kz, f2, g2, ref2);
+            pull<STO, R, int64_t, LAY, DEP>(c, A, plane, 2, kz, f2, g2, ref2);
             const R T1 = (c.T0 + reff) + dTf;
             const R T2 = (c.T0 + ref2) + (((g2[0] + g2[1]) + (g2[2] + g2[3])) + g2[4]);
             const R G = (kz >= c.hz0 && kz <= c.hz1) ? c.hG : R(0);
@@ -342,27 +353,27 @@ __device__ __forceinline__ void update_column(const Consts<float>& c, const Buf<
 // when the row's first element index is even (VEC: nz even, kz0 even); the shifted
 // columns of the e_z = +-1 populations are two scalar loads.  Flow populations carry the
 // flow reference: the pull adds D_pop(Q(source)), the store subtracts D_i(Q(own)).
-__device__ __forceinline__ V2 ld2(const __half* p, int a, int b, bool vec) {
-    if (vec) return {__half22float2(__ldg(reinterpret_cast<const __half2*>(p + a)))};
-    return v2(__half2float(__ldg(p + a)), __half2float(__ldg(p + b)));
+template <bool DEP = false> __device__ __forceinline__ V2 ld2(const __half* p, int a, int b, bool vec) {
+    if (vec) return {__half22float2(ld1<DEP>(reinterpret_cast<const __half2*>(p + a)))};
+    return v2(ldv<DEP>(p + a), ldv<DEP>(p + b));
 }
-__device__ __forceinline__ V2 ld2(const __nv_bfloat16* p, int a, int b, bool vec) {
-    if (vec) return {__bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162*>(p + a)))};
-    return v2(__bfloat162float(__ldg(p + a)), __bfloat162float(__ldg(p + b)));
+template <bool DEP = false> __device__ __forceinline__ V2 ld2(const __nv_bfloat16* p, int a, int b, bool vec) {
+    if (vec) return {__bfloat1622float2(ld1<DEP>(reinterpret_cast<const __nv_bfloat162*>(p + a)))};
+    return v2(ldv<DEP>(p + a), ldv<DEP>(p + b));
 }
-__device__ __forceinline__ V2 ld2(const float* p, int a, int b, bool vec) {
-    if (vec) return {__ldg(reinterpret_cast<const float2*>(p + a))};
-    return v2(__ldg(p + a), __ldg(p + b));
+template <bool DEP = false> __device__ __forceinline__ V2 ld2(const float* p, int a, int b, bool vec) {
+    if (vec) return {ld1<DEP>(reinterpret_cast<const float2*>(p + a))};
+    return v2(ldv<DEP>(p + a), ldv<DEP>(p + b));
 }
-__device__ __forceinline__ Q2 ldq2(const uint2* q, int a, int b, bool vec) {
+template <bool DEP = false> __device__ __forceinline__ Q2 ldq2(const uint2* q, int a, int b, bool vec) {
     uint2 ua, ub;
     if (vec) {
-        const uint4 u = __ldg(reinterpret_cast<const uint4*>(q + a));
+        const uint4 u = ld1<DEP>(reinterpret_cast<const uint4*>(q + a));
         ua = make_uint2(u.x, u.y);
         ub = make_uint2(u.z, u.w);
     } else {
-        ua = __ldg(q + a);
-        ub = __ldg(q + b);
+        ua = ld1<DEP>(q + a);
+        ub = ld1<DEP>(q + b);
     }
     const Qf x = fref_unpack(ua), y = fref_unpack(ub);
     return {v2(x.A, y.A), v2(x.Jr, y.Jr), v2(x.Jz, y.Jz), v2(x.R, y.R)};
@@ -452,7 +463,7 @@ __device__ __forceinline__ void pair_finish(const Consts<float>& c, const Buf<ST
 // Update rows kr0 .. kr0 + rows - 1 (non-wall rows below nr) of the column pair starting
 // at the even column kz0.  VEC: nz is even, so every row's first element index is even
 // and the own-column pairs are aligned for vector loads and stores.
-template <int STO, bool VEC>
+template <int STO, bool VEC, bool DEP = false>
 __device__ __forceinline__ void update_pair(const Consts<float>& c, const Buf<STO>& A, const Buf<STO>& B,
                                             const float* __restrict__ phi, int plane, int kr0, int rows, int kz0) {
     static_assert(has_fref<STO>(), "the packed pair update serves 16-bit storage");
@@ -482,26 +493,26 @@ __device__ __forceinline__ void update_pair(const Consts<float>& c, const Buf<ST
         const int p1 = axis ? 3 : 1, p5 = axis ? 6 : 5, p8 = axis ? 7 : 8;
         // own (kz0, zc1), left (zm0, kz0) and right (zp0, zp1) columns of a row
         V2 fh[9], gh[5];
-        fh[0] = ld2(F, row + kz0, row + zc1, VEC);
-        fh[1] = ld2(F + p1 * plane, rowm + kz0, rowm + zc1, VEC);
-        fh[2] = ld2(F + 2 * plane, row + zm0, row + kz0, false);
-        fh[3] = ld2(F + 3 * plane, rowp + kz0, rowp + zc1, VEC);
-        fh[4] = ld2(F + 4 * plane, row + zp0, row + zp1, false);
-        fh[5] = ld2(F + p5 * plane, rowm + zm0, rowm + kz0, false);
-        fh[6] = ld2(F + 6 * plane, rowp + zm0, rowp + kz0, false);
-        fh[7] = ld2(F + 7 * plane, rowp + zp0, rowp + zp1, false);
-        fh[8] = ld2(F + p8 * plane, rowm + zp0, rowm + zp1, false);
-        gh[0] = ld2(G, row + kz0, row + zc1, VEC);
-        gh[1] = ld2(G + p1 * plane, rowm + kz0, rowm + zc1, VEC);
-        gh[2] = ld2(G + 2 * plane, row + zm0, row + kz0, false);
-        gh[3] = ld2(G + 3 * plane, rowp + kz0, rowp + zc1, VEC);
-        gh[4] = ld2(G + 4 * plane, row + zp0, row + zp1, false);
-        const V2 ph = ld2(phi, row + kz0, row + zc1, VEC);
+        fh[0] = ld2<DEP>(F, row + kz0, row + zc1, VEC);
+        fh[1] = ld2<DEP>(F + p1 * plane, rowm + kz0, rowm + zc1, VEC);
+        fh[2] = ld2<DEP>(F + 2 * plane, row + zm0, row + kz0, false);
+        fh[3] = ld2<DEP>(F + 3 * plane, rowp + kz0, rowp + zc1, VEC);
+        fh[4] = ld2<DEP>(F + 4 * plane, row + zp0, row + zp1, false);
+        fh[5] = ld2<DEP>(F + p5 * plane, rowm + zm0, rowm + kz0, false);
+        fh[6] = ld2<DEP>(F + 6 * plane, rowp + zm0, rowp + kz0, false);
+        fh[7] = ld2<DEP>(F + 7 * plane, rowp + zp0, rowp + zp1, false);
+        fh[8] = ld2<DEP>(F + p8 * plane, rowm + zp0, rowm + zp1, false);
+        gh[0] = ld2<DEP>(G, row + kz0, row + zc1, VEC);
+        gh[1] = ld2<DEP>(G + p1 * plane, rowm + kz0, rowm + zc1, VEC);
+        gh[2] = ld2<DEP>(G + 2 * plane, row + zm0, row + kz0, false);
+        gh[3] = ld2<DEP>(G + 3 * plane, rowp + kz0, rowp + zc1, VEC);
+        gh[4] = ld2<DEP>(G + 4 * plane, row + zp0, row + zp1, false);
+        const V2 ph = ld2<DEP>(phi, row + kz0, row + zc1, VEC);
         const auto qw = [&](int rs, int cs) {   // words of row kr - 1 + rs, columns left / own / right
             const int r = rs == 0 ? rowm : (rs == 1 ? row : rowp);
-            if (cs == 1) return ldq2(Qp, r + kz0, r + zc1, VEC);
-            if (cs == 0) return ldq2(Qp, r + zm0, r + kz0, false);
-            return ldq2(Qp, r + zp0, r + zp1, false);
+            if (cs == 1) return ldq2<DEP>(Qp, r + kz0, r + zc1, VEC);
+            if (cs == 0) return ldq2<DEP>(Qp, r + zm0, r + kz0, false);
+            return ldq2<DEP>(Qp, r + zp0, r + zp1, false);
         };
         pair_finish<STO, VEC>(c, B, plane, kr, row, kz0, p1, p5, p8, fh, gh, ph, qw, st0, st1);
     }

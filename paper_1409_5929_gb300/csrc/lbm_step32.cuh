@@ -55,8 +55,8 @@ __device__ __forceinline__ bool pull_pair(const Consts32& c, const State32& A, c
     const float* __restrict__ F = A.f;
     const float* __restrict__ G = A.g;
     const auto own = [&](const float* p) { return ld_two<VEC>(p, kz, lb); };
-    const auto left = [&](const float* p) { return v2(__ldg(p + zm), __ldg(p + kz)); };
-    const auto right = [&](const float* p) { return v2(__ldg(p + zp0), __ldg(p + zp)); };
+    const auto left = [&](const float* p) { return v2(p[zm], p[kz]); };
+    const auto right = [&](const float* p) { return v2(p[zp0], p[zp]); };
     v.f[0] = own(F + row);
     v.f[1] = own(F + (i1 * plane + rowm));
     v.f[2] = left(F + (2 * plane + row));
@@ -73,7 +73,7 @@ __device__ __forceinline__ bool pull_pair(const Consts32& c, const State32& A, c
     v.g[4] = right(G + (4 * plane + row));
     v.ph = own(phi + row);
     const auto ref = [&](int o, int a, int b) {
-        return v2(__half2float(__ldg(c.tref + o + a)), __half2float(__ldg(c.tref + o + b)));
+        return v2(__half2float(c.tref[o + a]), __half2float(c.tref[o + b]));
     };
     v.R = ref_of(ld_ref<VEC>(c.tref + row, kz, lb));
     v.g[1] += (ref_of(ld_ref<VEC>(c.tref + rowm, kz, lb)) - v.R) * both(0.1f);
@@ -168,12 +168,12 @@ __device__ __forceinline__ void step_wall(const Consts32& c, const State32& A, c
     const int qm = q > 0 ? q - 1 : nz - 1, qp = q < nz - 1 ? q + 1 : 0;
     const int row = p * nz, rowp = row + nz, rowm = p == 0 ? row : row - nz, own = j * nz + z;
     const int i1 = p == 0 ? 3 : 1, i5 = p == 0 ? 6 : 5, i8 = p == 0 ? 7 : 8;
-    const auto f = [&](int i, int o) { return __ldg(A.f + i * plane + o); };
-    const auto g = [&](int i, int o) { return __ldg(A.g + i * plane + o); };
-    const auto ref = [&](int o) { return __half2float(__ldg(c.tref + o)); };
+    const auto f = [&](int i, int o) { return A.f[i * plane + o]; };
+    const auto g = [&](int i, int o) { return A.g[i * plane + o]; };
+    const auto ref = [&](int o) { return __half2float(c.tref[o]); };
     float fh[9] = {f(0, row + q), f(i1, rowm + q), f(2, row + qm), f(3, rowp + q), f(4, row + qp),
                    f(i5, rowm + qm), f(6, rowp + qm), f(7, rowp + qp), f(i8, rowm + qp)};
-    const float R = ref(row + q), Rj = ref(own), ph = __ldg(phi + row + q), phj = __ldg(phi + own);
+    const float R = ref(row + q), Rj = ref(own), ph = phi[row + q], phj = phi[own];
     float gh[5] = {g(0, row + q), g(i1, rowm + q) + 0.1f * (ref(rowm + q) - R), g(2, row + qm) + 0.1f * (ref(row + qm) - R),
                    g(3, rowp + q) + 0.1f * (ref(rowp + q) - R), g(4, row + qp) + 0.1f * (ref(row + qp) - R)};
     float lin, nl, iph, rho, ur, uz, dT;

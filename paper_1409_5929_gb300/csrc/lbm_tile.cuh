@@ -115,12 +115,12 @@ __device__ __forceinline__ void tile_steps(const Consts32& c, const State32& A, 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (int n = threadIdx.x; n < RN; n += blockDim.x) {
         const int y = n / RZ, x = n - y * RZ, g = (ra + y) * nz + wrap(za + x);
-        sR[n] = __half2float(__ldg(c.tref + g));
-        sP[n] = __ldg(phi + g);
+        sR[n] = __half2float(c.tref[g]);
+        sP[n] = phi[g];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) s0[i * RN + n] = __ldg(A.f + i * plane + g);
+        for (int i = 0; i < 9; ++i) s0[i * RN + n] = A.f[i * plane + g];
 #pragma unroll
-        for (int i = 0; i < 5; ++i) s0[(9 + i) * RN + n] = __ldg(A.g + i * plane + g);
+        for (int i = 0; i < 5; ++i) s0[(9 + i) * RN + n] = A.g[i * plane + g];
     }
     __syncthreads();
     // this thread's node (j, z)

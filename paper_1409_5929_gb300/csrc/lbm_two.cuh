@@ -317,8 +317,8 @@ __device__ __forceinline__ void wall_pair(const Consts32& c, int p, int j, int c
 
 // Two columns of a plane (VEC: aligned neighbours), and the stores of both or the first.
 template <bool VEC> __device__ __forceinline__ V2 ld_two(const float* p, int la, int lb) {
-    if (VEC) return {__ldg(reinterpret_cast<const float2*>(p + la))};
-    return v2(__ldg(p + la), __ldg(p + lb));
+    if (VEC) return {*reinterpret_cast<const float2*>(p + la)};
+    return v2(p[la], p[lb]);
 }
 template <bool VEC> __device__ __forceinline__ void st_two(float* p, V2 v, bool second) {
     if (VEC) {
@@ -330,9 +330,9 @@ template <bool VEC> __device__ __forceinline__ void st_two(float* p, V2 v, bool 
 }
 // Two columns of the reference plane R(x), as loaded and as floats.
 template <bool VEC> __device__ __forceinline__ uint32_t ld_ref(const __half* p, int la, int lb) {
-    if (VEC) return __ldg(reinterpret_cast<const uint32_t*>(p + la));
+    if (VEC) return *reinterpret_cast<const uint32_t*>(p + la);
     const auto* q = reinterpret_cast<const unsigned short*>(p);
-    return (uint32_t)__ldg(q + la) | ((uint32_t)__ldg(q + lb) << 16);
+    return (uint32_t)q[la] | ((uint32_t)q[lb] << 16);
 }
 __device__ __forceinline__ V2 ref_of(uint32_t w) { return {__half22float2(*reinterpret_cast<const __half2*>(&w))}; }
 
