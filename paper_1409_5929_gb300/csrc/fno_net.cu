@@ -61,7 +61,9 @@ __device__ int g_net_error;
 // first lets its own successor be scheduled and then waits until its predecessor has
 // completed and its writes are visible, before touching global or tensor memory.  The
 // successor is scheduled only once every CTA of this grid has started, so a kernel of
-// several waves is never short of SMs for its own CTAs.
+// several waves is never short of SMs for its own CTAs.  Inputs are no const __restrict__
+// parameters: the kernel is resident while earlier launches still write them, and the compiler
+// may turn such a parameter's loads into read-only ones, which nothing keeps behind the wait.
 __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -150,7 +152,7 @@ __device__ __forceinline__ void recover(const uint64_t* mbar, const uint32_t* ph
 }
 
 // ------------------------------------------------------------------- pack --
-__global__ void k_pack(const float* __restrict__ src, int64_t so, int64_t si, int O, int I, bf16* __restrict__ dst,
+__global__ void k_pack(const float* src, int64_t so, int64_t si, int O, int I, bf16* __restrict__ dst,
                        int Opad, int Ipad) {
     pdl_enter();
     const int64_t n = (int64_t)Opad * Ipad;
@@ -874,7 +876,7 @@ __global__ void __launch_bounds__(256, 2) k_bwd(const BwdP a) {
 // k_r2k: CTA (b, kz): out[kz][kr][part][b][:] = F2 [Z_re; Z_im], F2 (4M x 2 nr) padded to
 // 128 rows.  k_k2r: CTA (b, kz, row tile): out[b][kz][part][r][:] = F2i [Y_re; Y_im].
 template <int C>
-__global__ void __launch_bounds__(128) k_r2k(const bf16* __restrict__ in, const bf16* __restrict__ f2,
+__global__ void __launch_bounds__(128) k_r2k(const bf16* in, const bf16* f2,
                                              float* __restrict__ out, int B, int nr, int M) {
     pdl_enter();
     const int K = 2 * nr, kz = blockIdx.x % M, b = blockIdx.x / M;
@@ -932,7 +934,7 @@ __global__ void __launch_bounds__(128) k_r2k(const bf16* __restrict__ in, const 
 }
 
 template <int C>
-__global__ void __launch_bounds__(128) k_k2r(const float* __restrict__ in, const bf16* __restrict__ f2i,
+__global__ void __launch_bounds__(128) k_k2r(const float* in, const bf16* f2i,
                                              bf16* __restrict__ out, int B, int nr, int M) {
     pdl_enter();
     const int K = 4 * M, ntm = 2 * nr / 128;
@@ -997,7 +999,7 @@ __global__ void __launch_bounds__(128) k_k2r(const float* __restrict__ in, const
 // per thread took six.  Batch 8, C = 32, 16 modes: k_mixf 6.2 -> 4.9 us, k_mixb 12.6 -> 7.5 us.
 __host__ __device__ __forceinline__ int mix_pad(int B) { return (B + 3) & ~3; }   // batch in fours
 
-__global__ void k_mixf(const float* __restrict__ W, const float* __restrict__ R, float* __restrict__ Y, int B, int C,
+__global__ void k_mixf(const float* W, const float* R, float* __restrict__ Y, int B, int C,
                        int M) {
     pdl_enter();
     extern __shared__ __align__(16) float s[];
@@ -1039,7 +1041,7 @@ __global__ void k_mixf(const float* __restrict__ W, const float* __restrict__ R,
     }
 }
 
-__global__ void k_mixb(const float* __restrict__ W, const float* __restrict__ R, const float* __restrict__ dY,
+__global__ void k_mixb(const float* W, const float* R, const float* dY,
                        float* __restrict__ dW, float* __restrict__ dR, int B, int C, int M, int accumulate) {
     pdl_enter();
     extern __shared__ __align__(16) float s[];

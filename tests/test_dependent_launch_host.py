@@ -36,6 +36,7 @@ def _dependent_kernels(text):
 @pytest.mark.parametrize("name,kernels", [
     ("lbm_f32.cu", {"k_two", "k_step", "k_fields", "k_batch_step", "k_tile"}),
     ("lbm_16.cu", {"k_step16", "k_fields16", "k_batch_step16"}),
+    ("fno_net.cu", {"k_pack", "k_pack_many", "k_fwd", "k_proj", "k_bwd", "k_r2k", "k_k2r", "k_mixf", "k_mixb"}),
 ])
 def test_no_read_only_parameters(name, kernels):
     found = {}
@@ -46,7 +47,8 @@ def test_no_read_only_parameters(name, kernels):
     assert not any(found.values()), found
 
 
-@pytest.mark.parametrize("name", ["lbm_two.cuh", "lbm_step32.cuh", "lbm_tile.cuh", "lbm_f32.cu", "lbm_16.cu"])
+@pytest.mark.parametrize("name", ["lbm_two.cuh", "lbm_step32.cuh", "lbm_tile.cuh", "lbm_f32.cu", "lbm_16.cu",
+                                  "fno_net.cu", "tc.cuh"])
 def test_no_read_only_loads(name):
     assert "__ldg(" not in _source(name) and "ld.global.nc" not in _source(name)
 
