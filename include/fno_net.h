@@ -116,7 +116,7 @@ int fno_net_k2r(const fno_net_dims *d, const float *in, const void *f2i_img, voi
 
 /* Per-mode complex channel mixing Y = W R (each (kr, kz): [batch][C] x [C][C]) and its
  * backward: dW = dY R^H (overwritten), dR (+)= W^H dY summed over the batch
- * (accumulate = 1 adds). */
+ * (accumulate = 1 adds).  Any array may start at any float (16-byte alignment is faster). */
 int fno_net_mix_fwd(const fno_net_dims *d, const float *W, const float *R, float *Y, void *stream);
 int fno_net_mix_bwd(const fno_net_dims *d, const float *W, const float *R, const float *dY, float *dW, float *dR,
                     int accumulate, void *stream);

@@ -999,6 +999,13 @@ __global__ void __launch_bounds__(128) k_k2r(const float* in, const bf16* f2i,
 // per thread took six.  Batch 8, C = 32, 16 modes: k_mixf 6.2 -> 4.9 us, k_mixb 12.6 -> 7.5 us.
 __host__ __device__ __forceinline__ int mix_pad(int B) { return (B + 3) & ~3; }   // batch in fours
 
+// ALN: the caller's arrays (R and dR 8-byte aligned, W and dY of the backward and R of the forward
+// 16-byte aligned) allow wide accesses.  They need not: parameters sit one behind another in one
+// buffer, so those launches take single floats (a test of the pointers in the kernel cost a training
+// step 4 us of 465).
+static bool aligned(const float* p, int bytes) { return ((uintptr_t)p & (bytes - 1)) == 0; }
+
+template <bool ALN>
 __global__ void k_mixf(const float* W, const float* R, float* __restrict__ Y, int B, int C,
                        int M) {
     pdl_enter();
@@ -1007,9 +1014,14 @@ __global__ void k_mixf(const float* W, const float* R, float* __restrict__ Y, in
     float2* sR = reinterpret_cast<float2*>(s);   // [c][o]
     float* sX = s + 2 * C * C;                   // [part][c][b], b padded with zeros
     const int kz = blockIdx.x / (2 * M), kr = blockIdx.x % (2 * M);
-    const float4* Rm = reinterpret_cast<const float4*>(R + ((int64_t)kr * M + kz) * C * C * 2);
     const float* Wm = W + ((int64_t)kz * 2 * M + kr) * 2 * B * C;
-    for (int i = threadIdx.x; i < C * C / 2; i += blockDim.x) reinterpret_cast<float4*>(sR)[i] = Rm[i];
+    const float* Rm = R + ((int64_t)kr * M + kz) * C * C * 2;
+    if constexpr (ALN) {
+        for (int i = threadIdx.x; i < C * C / 2; i += blockDim.x)
+            reinterpret_cast<float4*>(sR)[i] = reinterpret_cast<const float4*>(Rm)[i];
+    } else {
+        for (int i = threadIdx.x; i < 2 * C * C; i += blockDim.x) s[i] = Rm[i];
+    }
     for (int i = threadIdx.x; i < 2 * B4 * C; i += blockDim.x) {
         const int c = i % C, pb = i / C, part = pb / B4, b = pb - part * B4;
         sX[(part * C + c) * B4 + b] = b < B ? Wm[(part * B + b) * C + c] : 0.f;
@@ -1041,6 +1053,7 @@ __global__ void k_mixf(const float* W, const float* R, float* __restrict__ Y, in
     }
 }
 
+template <bool ALN>
 __global__ void k_mixb(const float* W, const float* R, const float* dY,
                        float* __restrict__ dW, float* __restrict__ dR, int B, int C, int M, int accumulate) {
     pdl_enter();
@@ -1050,11 +1063,19 @@ __global__ void k_mixb(const float* W, const float* R, const float* dY,
     float2* sR = reinterpret_cast<float2*>(sY + 2 * B * C);   // [o][c], rows of C + 1
     const int kz = blockIdx.x / (2 * M), kr = blockIdx.x % (2 * M);
     const int64_t mode = (int64_t)kr * M + kz, slab = ((int64_t)kz * 2 * M + kr) * 2 * B * C;
-    const float2* Rm = reinterpret_cast<const float2*>(R + mode * C * C * 2);
-    for (int i = threadIdx.x; i < C * C; i += blockDim.x) sR[(i % C) * (C + 1) + i / C] = Rm[i];
-    for (int i = threadIdx.x; i < B * C / 2; i += blockDim.x) {   // (2 B C floats, C a multiple of 32)
-        reinterpret_cast<float4*>(sX)[i] = reinterpret_cast<const float4*>(W + slab)[i];
-        reinterpret_cast<float4*>(sY)[i] = reinterpret_cast<const float4*>(dY + slab)[i];
+    const float* Rm = R + mode * C * C * 2;
+    for (int i = threadIdx.x; i < C * C; i += blockDim.x)
+        sR[(i % C) * (C + 1) + i / C] = ALN ? reinterpret_cast<const float2*>(Rm)[i] : make_float2(Rm[2 * i], Rm[2 * i + 1]);
+    if constexpr (ALN) {
+        for (int i = threadIdx.x; i < B * C / 2; i += blockDim.x) {   // (2 B C floats, C a multiple of 32)
+            reinterpret_cast<float4*>(sX)[i] = reinterpret_cast<const float4*>(W + slab)[i];
+            reinterpret_cast<float4*>(sY)[i] = reinterpret_cast<const float4*>(dY + slab)[i];
+        }
+    } else {
+        for (int i = threadIdx.x; i < 2 * B * C; i += blockDim.x) {
+            sX[i] = W[slab + i];
+            sY[i] = dY[slab + i];
+        }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < mix_pad(B) / 4 * C; i += blockDim.x) {   // dW = dY R^H
@@ -1097,14 +1118,19 @@ __global__ void k_mixb(const float* W, const float* R, const float* dY,
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            float2* d = reinterpret_cast<float2*>(dR) + mode * C * C + (c0 + k) * C + o;
+            float* d = dR + 2 * (mode * C * C + (c0 + k) * C + o);
             float2 v = make_float2(gr[k], gi[k]);
             if (accumulate) {
-                const float2 old = *d;
+                const float2 old = ALN ? *reinterpret_cast<const float2*>(d) : make_float2(d[0], d[1]);
                 v.x = old.x + gr[k];
                 v.y = old.y + gi[k];
             }
-            *d = v;
+            if constexpr (ALN) {
+                *reinterpret_cast<float2*>(d) = v;
+            } else {
+                d[0] = v.x;
+                d[1] = v.y;
+            }
         }
     }
 }
@@ -1348,8 +1374,9 @@ int fno_net_mix_fwd(const fno_net_dims* d, const float* W, const float* R, float
     if ((size_t)(2 * C * C + 2 * B * C) * 4 > 200 * 1024)
         return fail(FNO_NET_ERR_INVALID, "fno_net_mix_fwd: batch too large");
     const size_t sb = (size_t)(2 * C * C + 2 * mix_pad(B) * C) * 4;
-    if (int rc = set_smem(k_mixf, sb)) return rc;
-    NCK(launch_pdl(k_mixf, dim3((unsigned)(2 * d->modes * d->modes)), dim3(256), sb, (cudaStream_t)stream, W, R, Y, B, C, d->modes));
+    const auto k = aligned(R, 16) ? k_mixf<true> : k_mixf<false>;
+    if (int rc = set_smem(k, sb)) return rc;
+    NCK(launch_pdl(k, dim3((unsigned)(2 * d->modes * d->modes)), dim3(256), sb, (cudaStream_t)stream, W, R, Y, B, C, d->modes));
     NCK(cudaGetLastError());
     return FNO_NET_OK;
 }
@@ -1363,8 +1390,10 @@ int fno_net_mix_bwd(const fno_net_dims* d, const float* W, const float* R, const
     if ((size_t)(2 * C * C + 4 * B * C) * 4 > 200 * 1024)
         return fail(FNO_NET_ERR_INVALID, "fno_net_mix_bwd: batch too large");
     const size_t sb = (size_t)(2 * C * (C + 1) + 4 * B * C) * 4;
-    if (int rc = set_smem(k_mixb, sb)) return rc;
-    NCK(launch_pdl(k_mixb, dim3((unsigned)(2 * d->modes * d->modes)), dim3(256), sb, (cudaStream_t)stream, W, R, dY, dW, dR, B, C, d->modes,
+    const bool wide = aligned(W, 16) && aligned(dY, 16) && aligned(R, 8) && aligned(dR, 8);
+    const auto k = wide ? k_mixb<true> : k_mixb<false>;
+    if (int rc = set_smem(k, sb)) return rc;
+    NCK(launch_pdl(k, dim3((unsigned)(2 * d->modes * d->modes)), dim3(256), sb, (cudaStream_t)stream, W, R, dY, dW, dR, B, C, d->modes,
                                                                                      accumulate));
     NCK(cudaGetLastError());
     return FNO_NET_OK;
