@@ -292,15 +292,15 @@ int lbm_get_info(lbm_handle *h, lbm_info *out);
 
 /* Bounded waits of the staged 16-bit bulk kernel (not an operation of the paper).  With
  * 16-bit storage, even nz and large grids (more than eight million nodes; at least 16 blocks
- * per SM once a limit was set here), the bulk step copies
+ * per SM once a limit, of any value, was set here), the bulk step copies
  * each row's source segments into shared memory with bulk copies whose completion every
  * thread awaits for at most `rounds` polls (default a few seconds).
  * A wait that runs out marks the handle: the block drains its copies in flight and
  * stops, so that step's results are invalid.  lbm_wait_status synchronises the handle's
  * stream and returns LBM_ERR_TIMEOUT if any wait ran out since the last clear (clear = 1
  * resets the mark), else LBM_OK; lbm_run checks it at every residual check.
- * lbm_set_wait_limit sets `rounds` (< 0: the default; 0 makes every wait run out at
- * once, for tests of the error path). */
+ * lbm_set_wait_limit sets `rounds` (< 0: the default, as if none had been set; 0 makes every
+ * wait run out at once, for tests of the error path). */
 int lbm_set_wait_limit(lbm_handle *h, int rounds);
 int lbm_wait_status(lbm_handle *h, int clear);
 /* enable = 0 runs the 16-bit bulk step on global loads everywhere (the update and its

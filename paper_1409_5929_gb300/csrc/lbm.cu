@@ -700,6 +700,7 @@ struct lbm_handle {
     std::vector<cudaEvent_t> ev;   // (bulk start, bulk end, wall start, wall end) per timed step
     int* wait_status = nullptr;    // 16-bit storage: LBM_ERR_TIMEOUT once a bounded wait of the staged kernel ran out
     int spin = STAGE_SPIN;         // try_wait rounds of its per-row waits
+    bool limit_set = false;        // by lbm_set_wait_limit, to any value
     int stage = 1;                 // 16-bit: the staged bulk kernel where it applies (lbm_set_staging)
     Plan32 plan = {};              // launches of several steps (FP32 storage, two buffers)
     Consts32 c32;
@@ -1244,7 +1245,7 @@ static int launch_step(lbm_handle* h) {
     constexpr int64_t STEP16_NODES = 8000000;
     const int64_t tiles16 = (int64_t)((h->p.nz + 2 * BULK_THREADS - 1) / (2 * BULK_THREADS)) * ((h->p.nr + BULK_RPT - 1) / BULK_RPT);
     const bool staged = h->stage && !(h->p.nz & 1) && tiles16 >= (int64_t)BULK_RPT_MIN_BLOCKS * h->sms &&
-                        (h->N > STEP16_NODES || h->spin != STAGE_SPIN);
+                        (h->N > STEP16_NODES || h->limit_set);
     if (h->step16 && !staged) {
         cudaEvent_t e[4] = {nullptr, nullptr, nullptr, nullptr};   // bulk start / end; no wall kernel
         if (h->timing) {
@@ -1677,6 +1678,7 @@ int lbm_set_staging(lbm_handle* h, int enable) {
 int lbm_set_wait_limit(lbm_handle* h, int rounds) {
     if (!h) return fail(LBM_ERR_INVALID, "handle is NULL");
     h->spin = rounds < 0 ? STAGE_SPIN : rounds;
+    h->limit_set = rounds >= 0;
     return LBM_OK;
 }
 
@@ -2135,6 +2137,7 @@ struct lbm_batch {
     size_t cap_stiles = 0;
     int* wait_status = nullptr;       // 16-bit: LBM_ERR_TIMEOUT once a bounded wait of k_batch_stage ran out
     int spin = STAGE_SPIN;            // try_wait rounds of its per-row waits
+    bool limit_set = false;           // by lbm_batch_set_wait_limit, to any value
     int stage = 1;                    // 16-bit: staged tiles for the even-nz instances (lbm_batch_set_staging)
     int sms = 0;                      // multiprocessors of the device
     // one launch per step (lbm_16.h)
@@ -2221,7 +2224,7 @@ static int batch_rebuild(lbm_batch* b) {
     Blocks16 sb16;
     int64_t nodes = 0;
     for (int i : act) nodes += (int64_t)b->p[i].nr * b->p[i].nz;
-    b->step16 = b->storage != LBM_F32 && (!b->stage || (nodes <= BATCH_STEP16_NODES && b->spin == STAGE_SPIN));
+    b->step16 = b->storage != LBM_F32 && (!b->stage || (nodes <= BATCH_STEP16_NODES && !b->limit_set));
     if (b->step16) {
         sb16 = blocks16(b->p, act);
         b->nblocks16[0] = (int)sb16.even.size();
@@ -2817,6 +2820,7 @@ int lbm_batch_set_staging(lbm_batch* b, int enable) {
 int lbm_batch_set_wait_limit(lbm_batch* b, int rounds) {
     if (!b) return fail(LBM_ERR_INVALID, "batch is NULL");
     b->spin = rounds < 0 ? STAGE_SPIN : rounds;
+    b->limit_set = rounds >= 0;
     return batch_rebuild(b);   // the launches (and the captured graph) follow the limit
 }
 
