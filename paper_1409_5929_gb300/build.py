@@ -22,7 +22,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 TARGETS = {
     "liblbm.so": ([os.path.join(CSRC, "lbm.cu"), os.path.join(CSRC, "lbm_f32.cu"),
                    os.path.join(CSRC, "lbm_16.cu")],
-                  [os.path.join(CSRC, n) for n in ("lbm_physics.cuh", "lbm_pair.cuh", "lbm_nodes.cuh", "lbm_dependent.h", "lbm_16.h", "lbm_f32.h", "lbm_two.cuh",
+                  [os.path.join(CSRC, n) for n in ("lbm_physics.cuh", "lbm_pair.cuh", "lbm_nodes.cuh", "lbm_dependent.h", "lbm_lists.h", "lbm_16.h", "lbm_f32.h", "lbm_two.cuh",
                                                    "lbm_tile.cuh", "lbm_step32.cuh")] + [os.path.join(INC, "lbm.h")]),
     "libfno.so": ([os.path.join(CSRC, "fno.cu")], [os.path.join(INC, "fno.h")]),
     "libfnonet.so": ([os.path.join(CSRC, "fno_net.cu")], [os.path.join(CSRC, "tc.cuh"), os.path.join(INC, "fno_net.h")]),

@@ -40,6 +40,7 @@
 #include "../../include/lbm.h"
 #include "lbm_16.h"
 #include "lbm_f32.h"
+#include "lbm_lists.h"
 #include "lbm_nodes.cuh"
 #include "lbm_pair.cuh"
 #include "lbm_physics.cuh"
@@ -2121,20 +2122,17 @@ struct lbm_batch {
     std::vector<char> active;         // 1 = still stepping
     // tiles and wall lists of the active set
     int bz = 128, rows = 1, rpt = 1;  // bulk block shape and rows per thread
-    int4* d_tiles = nullptr;          // active instances, all rows
+    DeviceList tiles;                 // int4: active instances, all rows
     int ntiles = 0;
     int ntiles_even = 0;              // leading tiles of instances with even nz
-    int* d_active = nullptr;
-    int* d_prefix = nullptr;
+    DeviceList act, prefix;           // int: active instances, their first wall threads
     int nactive = 0;
     int nwall = 0;
-    size_t cap_tiles = 0;
     double* partials = nullptr;
     double* result = nullptr;
     std::vector<int> iparity;         // buffer holding the state of an instance that stopped
-    int4* d_stiles = nullptr;         // 16-bit: staged tiles of the active instances with even nz
+    DeviceList stiles;                // int4, 16-bit: staged tiles of the active instances with even nz
     int nstiles = 0;
-    size_t cap_stiles = 0;
     int* wait_status = nullptr;       // 16-bit: LBM_ERR_TIMEOUT once a bounded wait of k_batch_stage ran out
     int spin = STAGE_SPIN;            // try_wait rounds of its per-row waits
     bool limit_set = false;           // by lbm_batch_set_wait_limit, to any value
@@ -2144,16 +2142,14 @@ struct lbm_batch {
     std::vector<Step16> inst16;
     std::vector<Inst32> inst32;
     Step16* d_inst16 = nullptr;
-    int2* d_blocks16 = nullptr;       // of the active instances: even nz, then odd nz
+    DeviceList blocks16;              // int2, of the active instances: even nz, then odd nz
     int nblocks16[2] = {0, 0};
     bool step16 = false;              // it serves the active instances
-    size_t cap_blocks16 = 0;
     // one launch per step (lbm_f32.h), where it serves every instance
     bool step32 = false;
     Inst32* d_inst32 = nullptr;
-    int2* d_blocks32 = nullptr;       // of the active instances: even nz, then odd nz
+    DeviceList blocks32;              // int2, of the active instances: even nz, then odd nz
     int nblocks32[2] = {0, 0};
-    size_t cap_blocks32 = 0;
     cudaGraphExec_t graph = nullptr;
     int64_t graph_steps = 0;
     int graph_parity = 0;             // batch parity the graph was captured at
@@ -2202,7 +2198,7 @@ static int batch_rebuild(lbm_batch* b) {
         for (int kr = 0; kr < b->p[i].nr; kr += b->rows * b->rpt)
             for (int z0 = 0; z0 < b->p[i].nz; z0 += zstep) dst.push_back(make_int4(i, kr, z0, 0));
     }
-    b->ntiles_even = (int)tiles.size();
+    const int tiles_even = (int)tiles.size();
     tiles.insert(tiles.end(), odd.begin(), odd.end());
     std::vector<int4> st;
     if (b->storage != LBM_F32 && b->stage) {
@@ -2212,65 +2208,34 @@ static int batch_rebuild(lbm_batch* b) {
                 for (int kr = 0; kr < b->p[i].nr; kr += rpt)
                     for (int z0 = 0; z0 < b->p[i].nz; z0 += 2 * BATCH_STAGE_NT) st.push_back(make_int4(i, kr, z0, rpt));
     }
-    b->nstiles = (int)st.size();
-    if (st.size() > b->cap_stiles) {
-        cudaFree(b->d_stiles);
-        b->d_stiles = nullptr;
-        CK(cudaMalloc((void**)&b->d_stiles, st.size() * sizeof(int4)));
-        b->cap_stiles = st.size();
-    }
-    if (!st.empty())
-        CK(cudaMemcpyAsync(b->d_stiles, st.data(), st.size() * sizeof(int4), cudaMemcpyHostToDevice, b->stream));
-    Blocks16 sb16;
     int64_t nodes = 0;
     for (int i : act) nodes += (int64_t)b->p[i].nr * b->p[i].nz;
-    b->step16 = b->storage != LBM_F32 && (!b->stage || (nodes <= BATCH_STEP16_NODES && !b->limit_set));
-    if (b->step16) {
-        sb16 = blocks16(b->p, act);
-        b->nblocks16[0] = (int)sb16.even.size();
-        b->nblocks16[1] = (int)sb16.odd.size();
-        sb16.even.insert(sb16.even.end(), sb16.odd.begin(), sb16.odd.end());
-        if (sb16.even.size() > b->cap_blocks16) {
-            cudaFree(b->d_blocks16);
-            b->d_blocks16 = nullptr;
-            CK(cudaMalloc((void**)&b->d_blocks16, sb16.even.size() * sizeof(int2)));
-            b->cap_blocks16 = sb16.even.size();
-        }
-        if (!sb16.even.empty())
-            CK(cudaMemcpyAsync(b->d_blocks16, sb16.even.data(), sb16.even.size() * sizeof(int2), cudaMemcpyHostToDevice,
-                               b->stream));
-    }
-    StepBlocks sb;
-    if (b->step32) {
-        sb = blocks32(b->p, act);
-        b->nblocks32[0] = (int)sb.even.size();
-        b->nblocks32[1] = (int)sb.odd.size();
-        sb.even.insert(sb.even.end(), sb.odd.begin(), sb.odd.end());
-        if (sb.even.size() > b->cap_blocks32) {
-            cudaFree(b->d_blocks32);
-            b->d_blocks32 = nullptr;
-            CK(cudaMalloc((void**)&b->d_blocks32, sb.even.size() * sizeof(int2)));
-            b->cap_blocks32 = sb.even.size();
-        }
-        if (!sb.even.empty())
-            CK(cudaMemcpyAsync(b->d_blocks32, sb.even.data(), sb.even.size() * sizeof(int2), cudaMemcpyHostToDevice, b->stream));
-    }
+    const bool step16 = b->storage != LBM_F32 && (!b->stage || (nodes <= BATCH_STEP16_NODES && !b->limit_set));
+    Blocks16 sb16;
+    if (step16) sb16 = blocks16(b->p, act);
+    StepBlocks sb32;
+    if (b->step32) sb32 = blocks32(b->p, act);
+    const int n16[2] = {(int)sb16.even.size(), (int)sb16.odd.size()}, n32[2] = {(int)sb32.even.size(), (int)sb32.odd.size()};
+    sb16.even.insert(sb16.even.end(), sb16.odd.begin(), sb16.odd.end());
+    sb32.even.insert(sb32.even.end(), sb32.odd.begin(), sb32.odd.end());
+    const ListUpload lists[] = {{&b->tiles, tiles.data(), tiles.size() * sizeof(int4)},
+                                {&b->stiles, st.data(), st.size() * sizeof(int4)},
+                                {&b->blocks16, sb16.even.data(), sb16.even.size() * sizeof(int2)},
+                                {&b->blocks32, sb32.even.data(), sb32.even.size() * sizeof(int2)},
+                                {&b->act, act.data(), act.size() * sizeof(int)},
+                                {&b->prefix, prefix.data(), prefix.size() * sizeof(int)}};
+    CK(upload_lists(lists, 6, b->stream));
+    // the counts follow the contents
     b->ntiles = (int)tiles.size();
+    b->ntiles_even = tiles_even;
+    b->nstiles = (int)st.size();
+    b->step16 = step16;
+    for (int k = 0; k < 2; ++k) {
+        b->nblocks16[k] = n16[k];
+        b->nblocks32[k] = n32[k];
+    }
     b->nactive = (int)act.size();
     b->nwall = prefix.back();
-    if ((size_t)b->ntiles > b->cap_tiles) {
-        cudaFree(b->d_tiles);
-        b->d_tiles = nullptr;
-        CK(cudaMalloc((void**)&b->d_tiles, tiles.size() * sizeof(int4)));
-        b->cap_tiles = tiles.size();
-    }
-    if (b->ntiles)
-        CK(cudaMemcpyAsync(b->d_tiles, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice, b->stream));
-    if (b->nactive) {
-        CK(cudaMemcpyAsync(b->d_active, act.data(), act.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream));
-    }
-    CK(cudaMemcpyAsync(b->d_prefix, prefix.data(), prefix.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream));
-    CK(cudaStreamSynchronize(b->stream));
     batch_free_graph(b);
     return LBM_OK;
 }
@@ -2288,7 +2253,7 @@ static int batch_launch_rebase_flow(lbm_batch* b) {
     if (b->storage != LBM_F32 && b->nactive) {
         const dim3 blk(b->bz, b->rows);
         DISPATCH_STO16(b->storage, DISPATCH_RPT(b->rpt, k_batch_rebase_flow<S_, R_><<<b->ntiles, blk, 0, b->stream>>>(
-                                                            b->d_desc, b->pool, b->parity, b->d_tiles)));
+                                                            b->d_desc, b->pool, b->parity, (const int4*)b->tiles.dev)));
         CK(cudaGetLastError());
     }
     b->since_rebase = 0;
@@ -2303,7 +2268,7 @@ static int batch_launch_step(lbm_batch* b) {
     if (b->step16) {
         for (int odd = 0; odd < 2; ++odd)
             if (b->nblocks16[odd])
-                CK(launch_batch16(b->storage, b->d_inst16, b->d_blocks16 + (odd ? b->nblocks16[0] : 0), b->nblocks16[odd],
+                CK(launch_batch16(b->storage, b->d_inst16, (const int2*)b->blocks16.dev + (odd ? b->nblocks16[0] : 0), b->nblocks16[odd],
                                   odd != 0, b->parity, b->stream));
         b->parity ^= 1;
         b->since_rebase += 1;
@@ -2312,7 +2277,7 @@ static int batch_launch_step(lbm_batch* b) {
     if (b->step32) {
         for (int odd = 0; odd < 2; ++odd)
             if (b->nblocks32[odd])
-                CK(launch_batch32(b->d_inst32, b->d_blocks32 + (odd ? b->nblocks32[0] : 0), b->nblocks32[odd], odd != 0,
+                CK(launch_batch32(b->d_inst32, (const int2*)b->blocks32.dev + (odd ? b->nblocks32[0] : 0), b->nblocks32[odd], odd != 0,
                                   b->parity, b->stream));
         b->parity ^= 1;
         b->since_rebase += 1;
@@ -2323,20 +2288,20 @@ static int batch_launch_step(lbm_batch* b) {
     CK(cudaEventRecord(b->wfork, b->stream));
     CK(cudaStreamWaitEvent(b->wstream, b->wfork, 0));
     DISPATCH_STO(b->storage, k_batch_wall<S_><<<(b->nwall + 127) / 128, 128, 0, b->wstream>>>(
-                                 b->d_desc, b->pool, b->parity, b->d_active, b->d_prefix, b->nactive));
+                                 b->d_desc, b->pool, b->parity, (const int*)b->act.dev, (const int*)b->prefix.dev, b->nactive));
     CK(cudaGetLastError());
     const dim3 blk(b->bz, b->rows);
     if (b->storage == LBM_F32) {
         DISPATCH_RPT(b->rpt, k_batch_bulk<LBM_F32, R_, false><<<b->ntiles, blk, 0, b->stream>>>(
-                                 b->d_desc, b->pool, b->parity, b->d_tiles));
+                                 b->d_desc, b->pool, b->parity, (const int4*)b->tiles.dev));
     } else {
         const int ne = b->ntiles_even, no = b->ntiles - b->ntiles_even;
         if (b->nstiles)   // even nz: staged tiles
             DISPATCH_STO16(b->storage, k_batch_stage<S_><<<b->nstiles, BATCH_STAGE_NT, 0, b->stream>>>(
-                                           b->d_desc, b->pool, b->parity, b->d_stiles, b->spin, b->wait_status));
+                                           b->d_desc, b->pool, b->parity, (const int4*)b->stiles.dev, b->spin, b->wait_status));
         if (no)
             DISPATCH_STO16(b->storage, DISPATCH_RPT(b->rpt, k_batch_bulk<S_, R_, false><<<no, blk, 0, b->stream>>>(
-                                                                b->d_desc, b->pool, b->parity, b->d_tiles + ne)));
+                                                                b->d_desc, b->pool, b->parity, (const int4*)b->tiles.dev + ne)));
     }
     CK(cudaGetLastError());
     CK(cudaEventRecord(b->wjoin, b->wstream));
@@ -2363,15 +2328,10 @@ int lbm_batch_destroy(lbm_batch* b) {
     cudaFree(b->pool);
     cudaFree(b->macpool);
     cudaFree(b->fstage);
-    cudaFree(b->d_tiles);
-    cudaFree(b->d_stiles);
+    for (DeviceList* l : {&b->tiles, &b->stiles, &b->blocks16, &b->blocks32, &b->act, &b->prefix}) cudaFree(l->dev);
     cudaFree(b->d_inst32);
-    cudaFree(b->d_blocks32);
     cudaFree(b->d_inst16);
-    cudaFree(b->d_blocks16);
     cudaFree(b->wait_status);
-    cudaFree(b->d_active);
-    cudaFree(b->d_prefix);
     cudaFree(b->partials);
     cudaFree(b->result);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
@@ -2437,8 +2397,6 @@ int lbm_batch_create(const lbm_params* p, int32_t n, lbm_batch** out) {
         }
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->macpool, mac_off * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_desc, n * sizeof(InstDesc));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_active, n * sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_prefix, (n + 1) * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->partials, (size_t)n * BATCH_RB * RES_NV * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->result, (size_t)n * RES_NV * sizeof(double));
     if (e == cudaSuccess && b->storage != LBM_F32) {
@@ -2575,7 +2533,9 @@ int lbm_batch_init_fields(lbm_batch* b, int32_t i, const float* ur, const float*
     CK(cudaStreamSynchronize(b->stream));
     if (!b->active[i]) {
         b->active[i] = 1;
-        return batch_rebuild(b);
+        const int rc = batch_rebuild(b);
+        if (rc) b->active[i] = 0;   // the lists are as before
+        return rc;
     }
     return LBM_OK;
 }
@@ -2625,7 +2585,7 @@ static int batch_snapshot(lbm_batch* b, int slot) {
     // moments use all rows of the active instances: the bulk tiles cover them
     const dim3 blk(b->bz, b->rows);
     DISPATCH_STO(b->storage, DISPATCH_RPT(b->rpt, k_batch_moments<S_, R_><<<b->ntiles, blk, 0, b->stream>>>(
-                                                       b->d_desc, b->pool, b->macpool, b->parity, slot, b->d_tiles)));
+                                                       b->d_desc, b->pool, b->macpool, b->parity, slot, (const int4*)b->tiles.dev)));
     CK(cudaGetLastError());
     return LBM_OK;
 }
@@ -2646,7 +2606,7 @@ int lbm_batch_run(lbm_batch* b, int64_t max_steps, int64_t check_every, double t
         const int64_t k = std::min(check_every, max_steps - total);
         // reference refresh before every check interval, as lbm_run does
         if (b->step32) {
-            CK(launch_batch_rebase32(b->d_inst32, b->d_active, b->nactive, b->parity, b->stream));
+            CK(launch_batch_rebase32(b->d_inst32, (const int*)b->act.dev, b->nactive, b->parity, b->stream));
         } else if (b->storage == LBM_F32) {
             for (int i = 0; i < b->n; ++i)
                 if (b->active[i] && (rc = batch_rebase_one(b, i))) return rc;
@@ -2688,7 +2648,7 @@ int lbm_batch_run(lbm_batch* b, int64_t max_steps, int64_t check_every, double t
         if ((rc = lbm_batch_wait_status(b, 0))) return rc;   // before the residual reads an invalid state
         if ((rc = batch_snapshot(b, slot))) return rc;
         const dim3 grid(BATCH_RB, b->nactive);
-        k_batch_resid<<<grid, 256, 0, b->stream>>>(b->d_desc, b->macpool, slot, b->d_active, b->partials);
+        k_batch_resid<<<grid, 256, 0, b->stream>>>(b->d_desc, b->macpool, slot, (const int*)b->act.dev, b->partials);
         CK(cudaGetLastError());
         k_batch_resid_final<<<b->nactive, 256, 0, b->stream>>>(b->partials, BATCH_RB, b->result);
         CK(cudaGetLastError());
@@ -2699,6 +2659,7 @@ int lbm_batch_run(lbm_batch* b, int64_t max_steps, int64_t check_every, double t
         for (int i = 0; i < b->n; ++i)
             if (b->active[i]) act.push_back(i);
         bool changed = false;
+        const auto was_active = b->active;
         int diverged = -1;
         for (int j = 0; j < b->nactive; ++j) {
             const double* q = &s[(size_t)j * RES_NV];
@@ -2720,7 +2681,10 @@ int lbm_batch_run(lbm_batch* b, int64_t max_steps, int64_t check_every, double t
             }
         }
         slot ^= 1;
-        if (changed && (rc = batch_rebuild(b))) return rc;
+        if (changed && (rc = batch_rebuild(b))) {
+            b->active = was_active;   // the lists are as before
+            return rc;
+        }
         if (diverged >= 0) {
             if (steps_out) std::copy(done.begin(), done.end(), steps_out);
             if (res_out) std::copy(res.begin(), res.end(), res_out);
