@@ -386,14 +386,16 @@ int lbm_batch_moments(lbm_batch *b, int32_t i, float *rho, float *ur, float *uz,
 int lbm_batch_pipe_nusselt(lbm_batch *b, int32_t i, double *nu, int32_t nz);
 /* Autotuner: times `steps` steps for each bulk tile shape (columns x rows per block x
  * rows per thread; twelve shapes of at most 256 threads) and keeps the fastest; *cols and
- * *rows receive the tile's columns and rows, *ms_per_step its time per step.  The state
- * advances by the steps the tuning ran (2 warm-up steps + `steps` per shape; the batch's
- * step count in lbm_batch_get_info includes them). */
+ * *rows receive the tile's columns and rows, *ms_per_step its time per step.  Where the steps
+ * launch no such tile (FP32 batches without a discrete heater; 16-bit batches of at most eight
+ * million nodes, or without an odd-nz instance) only the present shape is timed and kept.
+ * The state advances by the steps the tuning ran (2 warm-up steps + `steps` per shape; the
+ * batch's step count in lbm_batch_get_info includes them). */
 int lbm_batch_tune(lbm_batch *b, int32_t steps, int32_t *cols, int32_t *rows, float *ms_per_step);
 /* lbm_set_wait_limit and lbm_wait_status for the batch's staged 16-bit bulk kernel
  * (instances with even nz of batches of more than eight million nodes, or of any batch once a
- * limit was set; the tuned tile shape then serves the odd-nz instances and the
- * reference refresh).  lbm_batch_run checks the status after every check interval. */
+ * limit was set; the tile shape then serves the odd-nz instances and the reference
+ * refresh).  lbm_batch_run checks the status after every check interval. */
 int lbm_batch_set_wait_limit(lbm_batch *b, int rounds);
 int lbm_batch_wait_status(lbm_batch *b, int clear);
 int lbm_batch_set_staging(lbm_batch *b, int enable);

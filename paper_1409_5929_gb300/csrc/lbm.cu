@@ -29,6 +29,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <array>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -2240,6 +2241,26 @@ static int batch_rebuild(lbm_batch* b) {
     return LBM_OK;
 }
 
+// Another block shape; on an error the lists and the shape are as before.
+static int batch_reshape(lbm_batch* b, int bz, int rows, int rpt) {
+    const int old[3] = {b->bz, b->rows, b->rpt};
+    b->bz = bz;
+    b->rows = rows;
+    b->rpt = rpt;
+    const int rc = batch_rebuild(b);
+    if (rc) {
+        b->bz = old[0];
+        b->rows = old[1];
+        b->rpt = old[2];
+    }
+    return rc;
+}
+
+// Whether a step launches bulk tiles of that shape (k_batch_bulk).
+static bool batch_bulk_tiles(const lbm_batch* b) {
+    return !b->step32 && !b->step16 && (b->storage == LBM_F32 || b->ntiles > b->ntiles_even);
+}
+
 template <int STO> static Buf<STO> batch_buf(const lbm_batch* b, int i, int which) {
     const InstDesc& d = b->desc[i];
     Buf<STO> r;
@@ -2771,7 +2792,8 @@ int lbm_batch_moments(lbm_batch* b, int32_t i, float* rho, float* ur, float* uz,
 
 // Autotuner: time `steps` batched steps for each bulk tile shape (columns x rows per
 // block x rows per thread, at most 256 threads) and keep the fastest.  Leaves the state
-// advanced by the steps it ran (2 warm-up + `steps` per shape).
+// advanced by the steps it ran (2 warm-up + `steps` per shape).  Steps that launch no such
+// tile (k_batch_step, k_batch_step16, staged tiles alone) time the present shape only.
 static const int kTuneShapes[][3] = {{64, 1, 1}, {128, 1, 1}, {256, 1, 1}, {64, 2, 1}, {128, 2, 1}, {64, 4, 1},
                                      {32, 8, 1}, {64, 1, 2}, {64, 1, 4}, {128, 1, 2}, {128, 1, 4}, {32, 4, 4}};
 
@@ -2811,11 +2833,13 @@ int lbm_batch_tune(lbm_batch* b, int32_t steps, int32_t* bz_out, int32_t* rows_o
     float best = INFINITY;
     int bb = b->bz, br = b->rows, bt = b->rpt;
     int rc = LBM_OK;
-    for (const auto& s : kTuneShapes) {
-        b->bz = s[0];
-        b->rows = s[1];
-        b->rpt = s[2];
-        if ((rc = batch_rebuild(b))) break;
+    std::vector<std::array<int, 3>> shapes;
+    if (batch_bulk_tiles(b))
+        for (const auto& s : kTuneShapes) shapes.push_back({s[0], s[1], s[2]});
+    else
+        shapes.push_back({bb, br, bt});
+    for (const auto& s : shapes) {
+        if (s != std::array<int, 3>{b->bz, b->rows, b->rpt} && (rc = batch_reshape(b, s[0], s[1], s[2]))) break;
         if ((rc = lbm_batch_step(b, 2))) break;   // warm-up
         cudaEventRecord(e0, b->stream);
         if ((rc = lbm_batch_step(b, steps))) break;
@@ -2828,10 +2852,7 @@ int lbm_batch_tune(lbm_batch* b, int32_t steps, int32_t* bz_out, int32_t* rows_o
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc) return rc;
-    b->bz = bb;
-    b->rows = br;
-    b->rpt = bt;
-    if ((rc = batch_rebuild(b))) return rc;
+    if ((bb != b->bz || br != b->rows || bt != b->rpt) && (rc = batch_reshape(b, bb, br, bt))) return rc;
     if (bz_out) *bz_out = bb;
     if (rows_out) *rows_out = br * bt;
     if (ms_out) *ms_out = best / (float)steps;
