@@ -2799,12 +2799,14 @@ static const int kTuneShapes[][3] = {{64, 1, 1}, {128, 1, 1}, {256, 1, 1}, {64, 
 
 int lbm_batch_set_staging(lbm_batch* b, int enable) {
     if (!b) return fail(LBM_ERR_INVALID, "batch is NULL");
+    CK(cudaSetDevice(b->device));
     b->stage = enable != 0;
     return batch_rebuild(b);   // the tile lists (and the captured graph) follow the choice
 }
 
 int lbm_batch_set_wait_limit(lbm_batch* b, int rounds) {
     if (!b) return fail(LBM_ERR_INVALID, "batch is NULL");
+    CK(cudaSetDevice(b->device));
     b->spin = rounds < 0 ? STAGE_SPIN : rounds;
     b->limit_set = rounds >= 0;
     return batch_rebuild(b);   // the launches (and the captured graph) follow the limit
