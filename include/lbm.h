@@ -184,7 +184,8 @@ int lbm_init_fields(lbm_handle *h, const float *ur, const float *uz, const float
 /* Advance nsteps >= 0 time steps (asynchronous on the handle's stream).  With FP32 storage
  * in two buffers (and no discrete heater) a launch holds the boundary nodes too, and on small
  * and on large grids several steps; the last step of a call is always a launch of its own, so
- * that the previous state is kept (lbm_residual). */
+ * that the previous state is kept (lbm_residual).  Under stream capture an even number of steps
+ * takes an even number of launches, so a replay starts where the one before it ended. */
 int lbm_step(lbm_handle *h, int64_t nsteps);
 
 /* Fields of the current state (what the next step's pull sees, after the wall

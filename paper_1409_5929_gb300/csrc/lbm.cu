@@ -1356,9 +1356,26 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
     if (!h) return fail(LBM_ERR_INVALID, "handle is NULL");
     if (nsteps < 0) return fail(LBM_ERR_INVALID, "nsteps < 0");
     CK(cudaSetDevice(h->device));
+    const bool many = h->plan.two.strips != 0;
+    // Launches alternate between the buffers.  A captured call is replayed on the buffers it was captured
+    // with, so it takes an even number of launches for an even number of steps: where the plan would not,
+    // its first launch is split.
+    bool split = false;
+    if (many && nsteps > 1) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess) (void)cudaGetLastError();
+        split = cap == cudaStreamCaptureStatusActive && ((launches32(h->plan, nsteps) ^ nsteps) & 1);
+    }
+    int rest = 0;   // of a split launch
     for (int64_t s = 0; s < nsteps;) {
-        const int n = h->plan.two.strips ? steps32(h->plan, nsteps - s) : 1;
-        const int rc = h->plan.two.strips ? launch_steps(h, n) : launch_step(h);
+        int n = rest ? rest : many ? steps32(h->plan, nsteps - s) : 1;
+        rest = 0;
+        if (split) {
+            rest = n - 1;
+            n = 1;
+            split = false;
+        }
+        const int rc = many ? launch_steps(h, n) : launch_step(h);
         if (rc) return rc;
         s += n;
     }

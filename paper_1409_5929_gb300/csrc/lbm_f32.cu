@@ -284,6 +284,12 @@ int steps32(const Plan32& w, int64_t left) {
     return w.two.strips && left >= 3 && !w.single ? 2 : 1;
 }
 
+int64_t launches32(const Plan32& w, int64_t n) {
+    int64_t k = 0;
+    for (; n > 0; ++k) n -= steps32(w, n);
+    return k;
+}
+
 cudaError_t launch32(const Plan32& w, const Consts32& c, const State32& A, const State32& B, const float* phi, int plane,
                      int steps, cudaStream_t stream) {
     if (w.tile.T)

@@ -65,6 +65,8 @@ cudaError_t plan32(const lbm_params& p, int sms, Plan32* out);
 // Steps the next launch takes when `left` remain.  The last launch of a run takes a single step: it
 // leaves the previous state in the other buffer.
 int steps32(const Plan32& w, int64_t left);
+// Launches that n steps take (as many as steps, or fewer if the first one takes more than one).
+int64_t launches32(const Plan32& w, int64_t n);
 cudaError_t launch32(const Plan32& w, const Consts32& c, const State32& A, const State32& B, const float* phi, int plane,
                      int steps, cudaStream_t stream);
 
