@@ -2644,7 +2644,10 @@ int lbm_batch_run(lbm_batch* b, int64_t max_steps, int64_t check_every, double t
         const int64_t k = std::min(check_every, max_steps - total);
         // reference refresh before every check interval, as lbm_run does
         if (b->step32) {
-            CK(launch_batch_rebase32(b->d_inst32, (const int*)b->act.dev, b->nactive, b->parity, b->stream));
+            int64_t most = 0;
+            for (int i = 0; i < b->n; ++i)
+                if (b->active[i]) most = std::max(most, (int64_t)b->p[i].nr * b->p[i].nz);
+            CK(launch_batch_rebase32(b->d_inst32, (const int*)b->act.dev, b->nactive, most, b->parity, b->stream));
         } else if (b->storage == LBM_F32) {
             for (int i = 0; i < b->n; ++i)
                 if (b->active[i] && (rc = batch_rebase_one(b, i))) return rc;

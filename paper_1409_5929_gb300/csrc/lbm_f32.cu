@@ -126,7 +126,9 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_STEP_MIN_BLOCKS) k_batch_ste
 
 // Reference refresh (rebase_thermal_node of lbm.cu) of the instances act[blockIdx.y]: R(x) becomes the
 // temperature offset of the state in buffer `which`, the stored temperatures are re-expressed against it.  One
-// launch for the batch: 16 launches of k_rebase took 73 us.
+// launch for the batch: 16 launches of k_rebase took 73 us.  Blocks per instance for four nodes per thread
+// of the largest one, as many as k_rebase's 4096 at most (64 each left most of the device idle on one or
+// two large instances: 1 x 4096 x 4096 8134 against 7573 us per check, 1 x 1500 x 3000 2192 against 2040).
 __global__ void __launch_bounds__(256) k_batch_rebase(const Inst32* __restrict__ inst, const int* __restrict__ act, int which) {
     const Inst32& d = inst[act[blockIdx.y]];
     const int N = d.c.nr * d.c.nz, plane = d.plane;
@@ -338,8 +340,10 @@ cudaError_t launch_fields32(const Consts32& c, const State32& A, const float* ph
                             walls, fields_of(c.nz, rho, ur, uz, T));
 }
 
-cudaError_t launch_batch_rebase32(const Inst32* inst, const int* act, int n, int which, cudaStream_t stream) {
-    k_batch_rebase<<<dim3(64, (unsigned)n), 256, 0, stream>>>(inst, act, which);
+cudaError_t launch_batch_rebase32(const Inst32* inst, const int* act, int n, int64_t most_nodes, int which,
+                                  cudaStream_t stream) {
+    const unsigned blocks = (unsigned)std::min<int64_t>((most_nodes + 1023) / 1024, 4096);
+    k_batch_rebase<<<dim3(blocks, (unsigned)n), 256, 0, stream>>>(inst, act, which);
     return cudaGetLastError();
 }
 

@@ -88,8 +88,10 @@ struct StepBlocks {
 };
 bool serves32(const lbm_params& p);   // FP32 storage, no discrete heater
 StepBlocks blocks32(const std::vector<lbm_params>& p, const std::vector<int>& act);
-// lbm_rebase of the instances act[0 .. n - 1] (device memory), state in buffer `which`.
-cudaError_t launch_batch_rebase32(const Inst32* inst, const int* act, int n, int which, cudaStream_t stream);
+// lbm_rebase of the instances act[0 .. n - 1] (device memory; most_nodes: of the largest), state in
+// buffer `which`.
+cudaError_t launch_batch_rebase32(const Inst32* inst, const int* act, int n, int64_t most_nodes, int which,
+                                  cudaStream_t stream);
 cudaError_t launch_batch32(const Inst32* inst, const int2* blocks, int n, bool odd_nz, int parity, cudaStream_t stream);
 
 }  // namespace lbm
