@@ -1290,14 +1290,10 @@ static int launch_step(lbm_handle* h) {
             if (h->p.nz % 8 == 0) k_bulk_stage<S_, BULK_RPT, true><<<gb, BULK_THREADS, 0, h->stream>>>(h->cf, A, B, ph, (int)h->plane, h->spin, h->wait_status);
             else k_bulk_stage<S_, BULK_RPT, false><<<gb, BULK_THREADS, 0, h->stream>>>(h->cf, A, B, ph, (int)h->plane, h->spin, h->wait_status);
         });
-    } else if (rpt > 1) {
-        DISPATCH_STO(h->p.storage,
-                     k_bulk<S_, int, BULK_RPT><<<gb, BULK_THREADS, 0, h->stream>>>(
-                         h->cf, bufp<S_>(h, h->cur), bufp<S_>(h, h->cur ^ 1), (const PP<S_>*)h->phi, (int)h->plane));
-    } else if (i32) {
-        DISPATCH_STO(h->p.storage,
-                     k_bulk<S_, int, 1><<<gb, BULK_THREADS, 0, h->stream>>>(
-                         h->cf, bufp<S_>(h, h->cur), bufp<S_>(h, h->cur ^ 1), (const PP<S_>*)h->phi, (int)h->plane));
+    } else if (i32) {   // FP32 storage with the discrete heater
+        const auto k = rpt > 1 ? k_bulk<LBM_F32, int, BULK_RPT> : k_bulk<LBM_F32, int, 1>;
+        k<<<gb, BULK_THREADS, 0, h->stream>>>(h->cf, bufp<LBM_F32>(h, h->cur), bufp<LBM_F32>(h, h->cur ^ 1),
+                                              (const float*)h->phi, (int)h->plane);
     } else {
         DISPATCH_STO(h->p.storage,
                      k_bulk<S_, int64_t, 1><<<gb, BULK_THREADS, 0, h->stream>>>(
@@ -1888,10 +1884,9 @@ template <int STO> __host__ __device__ constexpr int bulk_cols() { return has_fr
 #ifndef LBM_BATCH_DESC_SMEM
 #define LBM_BATCH_DESC_SMEM 1
 #endif
-// VEC (16-bit storage): every tile of the launch belongs to an instance with even nz, so
-// the pair update may use its vector loads; tiles of odd-nz instances go to a VEC = false
-// launch (batch_rebuild orders them last).
-template <int STO, int RPT, bool VEC>
+// 16-bit storage: the tiles of odd-nz instances (batch_rebuild orders them last), whose rows start at
+// alternating alignment, so the pair update takes single loads.
+template <int STO, int RPT>
 __global__ void __launch_bounds__(256) k_batch_bulk(const InstDesc* __restrict__ desc, char* __restrict__ pool,
                                                     int parity, const int4* __restrict__ tiles) {
     const int4 t = tiles[blockIdx.x];
@@ -1918,7 +1913,7 @@ __global__ void __launch_bounds__(256) k_batch_bulk(const InstDesc* __restrict__
     const typename St<STO>::P* phi = (const typename St<STO>::P*)(pool + d.off_phi);
     const int plane = (int)d.plane;
     if constexpr (has_fref<STO>()) {
-        update_pair<STO, VEC>(c, A, B, phi, plane, t.y + threadIdx.y * RPT, RPT, kz);
+        update_pair<STO, false>(c, A, B, phi, plane, t.y + threadIdx.y * RPT, RPT, kz);
     } else {
         update_column<STO, int>(c, A, B, phi, plane, t.y + threadIdx.y * RPT, RPT, kz);
     }
@@ -2205,7 +2200,7 @@ static int batch_stage_rows(const lbm_batch* b, const std::vector<int>& act) {
 // staged: its waits are what the limit is for.
 constexpr int64_t BATCH_STEP16_NODES = 8000000;
 static int batch_rebuild(lbm_batch* b) {
-    std::vector<int4> tiles, odd;   // tiles of instances with odd nz last (k_batch_bulk's VEC)
+    std::vector<int4> tiles, odd;   // tiles of instances with odd nz last (16-bit storage: k_batch_bulk's)
     std::vector<int> act, prefix(1, 0);
     for (int i = 0; i < b->n; ++i) {
         if (!b->active[i]) continue;
@@ -2330,7 +2325,7 @@ static int batch_launch_step(lbm_batch* b) {
     CK(cudaGetLastError());
     const dim3 blk(b->bz, b->rows);
     if (b->storage == LBM_F32) {
-        DISPATCH_RPT(b->rpt, k_batch_bulk<LBM_F32, R_, false><<<b->ntiles, blk, 0, b->stream>>>(
+        DISPATCH_RPT(b->rpt, k_batch_bulk<LBM_F32, R_><<<b->ntiles, blk, 0, b->stream>>>(
                                  b->d_desc, b->pool, b->parity, (const int4*)b->tiles.dev));
     } else {
         const int ne = b->ntiles_even, no = b->ntiles - b->ntiles_even;
@@ -2338,7 +2333,7 @@ static int batch_launch_step(lbm_batch* b) {
             DISPATCH_STO16(b->storage, k_batch_stage<S_><<<b->nstiles, BATCH_STAGE_NT, 0, b->stream>>>(
                                            b->d_desc, b->pool, b->parity, (const int4*)b->stiles.dev, b->spin, b->wait_status));
         if (no)
-            DISPATCH_STO16(b->storage, DISPATCH_RPT(b->rpt, k_batch_bulk<S_, R_, false><<<no, blk, 0, b->stream>>>(
+            DISPATCH_STO16(b->storage, DISPATCH_RPT(b->rpt, k_batch_bulk<S_, R_><<<no, blk, 0, b->stream>>>(
                                                                 b->d_desc, b->pool, b->parity, (const int4*)b->tiles.dev + ne)));
     }
     CK(cudaGetLastError());
