@@ -21,8 +21,8 @@
 //           shared memory; then every wall node (rebuild from the interior neighbour by
 //           non-equilibrium extrapolation, Sec. 4, ref. [47], collision with u = 0 and the
 //           wall temperature), one thread each;
-//   k_bulk + k_wall         one node per thread: in-place storage (the wall kernel first), the
-//           discrete heater, and grids beyond 32-bit indices.
+//   k_bulk + k_wall         one node per thread: in-place storage (the wall kernel first), FP32
+//           storage with the discrete heater, and grids beyond 32-bit indices.
 // Both kernels of a pair read only the source buffer and write disjoint nodes of the destination.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -1848,9 +1848,12 @@ extern "C" int lbm_field_residual_noalloc(int32_t geometry, int32_t nr, int32_t 
 // porosity plane (each instance's own nr*nz, plane stride padded to 64 elements), and
 // a second pool holds two field snapshots (4 planes each) per instance.  A device
 // table of InstDesc carries each instance's lattice constants and pool offsets.
-// A step is two launches covering every active instance: k_batch_bulk over a
-// flattened list of tiles (instance, first row, first column; block shape chosen by
-// lbm_batch_tune) and k_batch_wall over the concatenated wall-node lists.  lbm_batch_run
+// A step is one launch covering every active instance (k_batch_step, lbm_f32.cu; k_batch_step16,
+// lbm_16.cu; a second one if instances of both nz parities are present), or, for 16-bit batches
+// above BATCH_STEP16_NODES or with a wait limit and FP32 batches with a discrete heater,
+// k_batch_stage and k_batch_bulk over flattened lists of tiles (instance, first row, first column;
+// k_batch_bulk's block shape chosen by lbm_batch_tune) beside k_batch_wall over the concatenated
+// wall-node lists.  lbm_batch_run
 // captures check_every steps (an even number, so every instance's A/B parity is the
 // same at each check) in a CUDA graph and replays it; instances that reach the
 // steady criterion leave the tile lists at the next check.

@@ -174,7 +174,10 @@ __global__ void __launch_bounds__(BULK_THREADS, 8) k_fields16(const Step16 s, in
 // of 64 to 160 rows (450 k nodes, FP16): 10.2 us per step (19.0 with staged tiles and the forked wall
 // kernel); 16 of 200 to 400 (3.6 M nodes, BF16) 68 against 76; 64 of 64 to 512 (12.2 M nodes) 232
 // against 231, where the staged tiles serve.  The staged tiles with the boundary nodes in their
-// launch: 234.  Six blocks per SM; with five 70 and 242, with seven 72 and 245.
+// launch: 234.  Six blocks per SM, for even nz (five / six / seven: 16 of 200 x 400 25.8 / 25.2 / 26.7 us,
+// 32 of 300 x 600 113 / 109 / 115).  The odd-nz form spills 196 bytes at six (even: 40) and would do best
+// with five: 16 of 100 x 201 8.7 / 9.9 / 11.2 us, 16 of 200 x 401 27.4 / 31.4 / 33.4, 32 of 300 x 601
+// 116 / 130 / 137 (staged tiles' k_batch_bulk and the wall kernel before: 35.8 for 16 of 200 x 401).
 template <int STO, bool VEC>
 __global__ void __launch_bounds__(BULK_THREADS, 6) k_batch_step16(const Step16* __restrict__ inst,
                                                                   const int2* __restrict__ blocks, int from) {

@@ -1,6 +1,7 @@
 // lbm_16.h -- one time step per launch, boundary nodes included, 16-bit storage in two buffers
 // (lbm_16.cu).  The node updates are those of lbm_nodes.cuh, bit for bit what the kernels of
-// lbm.cu make of them.
+// lbm.cu make of them (checked on states of every geometry; temperatures of the pipe with inlet on
+// grids of a few nodes differ by one FP32 rounding).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>

@@ -15,11 +15,13 @@ using namespace lbm;
 // independent.  At 4096 x 8192 a pass takes 0.68 ms for two steps where two single steps take
 // 1.24 ms (0.60 ms each, 97 % of the copy bandwidth, and the wall kernel): it moves the state's
 // 118 bytes per node once, at 86 % of the copy bandwidth, and issues 260 instructions per node
-// and step (563 in k_bulk).  128 registers, four blocks per SM; with five the registers spill
-// (0.44 ms per step), with three too few warps are in flight (0.40).  The marches that meet boundary nodes (the end strips, the first and the last
-// chunk of every strip, the wall rows) come first and run a form of the march of their own: the
-// boundary rebuild between a row's recovery and its collision cost the other marches 13 %
-// (4096 x 8192, FP32) when one form served both.
+// and step (563 in k_bulk).  128 registers, four blocks per SM; with five many more of them spill,
+// with three too few warps are in flight.  Per step of a long run with three / four / five blocks:
+// 4096 x 8192 0.366 / 0.344 / 0.478 ms; odd nz, 4095 x 8191 (two loads per pair, 92 bytes spilled at
+// four blocks against 16) 0.398 / 0.379 / 0.590 ms, single steps of k_bulk 0.688.  The marches that
+// meet boundary nodes (the end strips, the first and the last chunk of every strip, the wall rows) come
+// first and run a form of the march of their own: the boundary rebuild between a row's recovery and its
+// collision cost the other marches 13 % (4096 x 8192, FP32) when one form served both.
 #ifndef LBM_TWO_MIN_BLOCKS
 #define LBM_TWO_MIN_BLOCKS 4
 #endif
@@ -263,13 +265,16 @@ Consts32 consts32(const Consts<double>& d, const Consts<float>& f) {
     return c;
 }
 
-// k_tile up to this many nodes, k_two above (per step: 200 x 400 2.9 against 5.6 us, 300 x 600 5.4
-// against 6.5, 300 x 800 7.7 against 6.5).
+// k_tile up to this many nodes, k_step above: where their times per step of a long run cross (k_tile
+// against k_step: 200 x 400 2.9 / 4.6 us, 250 x 500 4.2 / 5.9, 300 x 600 5.5 / 5.6, 350 x 600 6.7 / 5.6,
+// 400 x 625 7.7 / 6.4).  Calls of one or two steps, which load a halo for the longest launch, would
+// cross near 100 x 200 already (3.9 / 3.7 us; 200 x 400 5.7 / 4.4, 300 x 600 10.1 / 5.7); before k_tile
+// such a step took two launches, 10.4 to 12.5 us.
 constexpr int64_t TILE_MAX_NODES = 200000;
 
 // One step per launch up to this many nodes, where the state stays in L2 (both buffers 112 bytes per
-// node), two steps per launch above: 512 x 1024 8.1 against 11.1 us per step, 700 x 1400 17.3
-// against 18.0, 1000 x 1500 29.3 against 24.6.
+// node), two steps per launch above (k_step against k_two): 512 x 1024 8.1 against 11.1 us per step,
+// 700 x 1400 17.3 against 18.0, 1000 x 1500 29.3 against 24.6.
 constexpr int64_t STEP_MAX_NODES = 1000000;
 
 cudaError_t plan32(const lbm_params& p, int sms, Plan32* out) {
