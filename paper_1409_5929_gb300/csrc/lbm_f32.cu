@@ -89,9 +89,11 @@ __global__ void __launch_bounds__(STEP_THREADS, LBM_STEP_MIN_BLOCKS) k_step(cons
 }
 // The fields of a state (what the next step's pull sees).  Against k_moments (one node per thread and
 // the boundary rebuild in the same warps): one step of 48 x 96 and its fields 8.2 -> 7.1 us,
-// 4096 x 8192 0.42 -> 0.36 ms (FP16 storage, k_fields16: 0.48 -> 0.36).
+// 4096 x 8192 0.42 -> 0.36 ms (FP16 storage, k_fields16: 0.48 -> 0.36).  Blocks per SM 8 / 9 / 10 / 11:
+// 4096 x 8192 372 / 368 / 364 / 376 us, 512 x 1024 5.63 / 5.54 / 5.48 / 6.47; odd nz, 4095 x 8191
+// 394 / 389 / 398 / 432, 1023 x 2047 27.2 / 26.9 / 28.5 / 31.7.
 template <bool VEC>
-__global__ void __launch_bounds__(STEP_THREADS, 8) k_fields(const Consts32 c, const State32 A, const float* phi,
+__global__ void __launch_bounds__(STEP_THREADS, VEC ? 10 : 9) k_fields(const Consts32 c, const State32 A, const float* phi,
                                                             int plane, int walls, const Fields o) {
     const int wall_blocks = (walls + STEP_THREADS - 1) / STEP_THREADS;
     asm volatile("griddepcontrol.wait;" ::: "memory");
