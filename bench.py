@@ -41,9 +41,9 @@ E2E_STEPS = 50                    # minimum length of the end-to-end window (ste
 # DRAM traffic of one bulk launch (FP32: k_two, two steps) on the 4096 x 8192 workload (dram__bytes_read.sum +
 # dram__bytes_write.sum of the bulk kernel in one single-pass ncu capture of this
 # benchmark), valid only for the bulk kernel's source it was taken on (_kernel_hash).
-TRAFFIC = {("f32", 4096, 8192): ("255f586a56e33446", 2285157632 + 1841550336),
-           ("f16", 4096, 8192): ("255f586a56e33446", 1690624768 + 1227723520),
-           ("bf16", 4096, 8192): ("255f586a56e33446", 1689783808 + 1227624448)}
+TRAFFIC = {("f32", 4096, 8192): ("db094916e40bc044", 2284458496 + 1841697280),
+           ("f16", 4096, 8192): ("db094916e40bc044", 1690585600 + 1227648256),
+           ("bf16", 4096, 8192): ("db094916e40bc044", 1689783808 + 1227962624)}
 
 
 def _kernel_hash() -> str:
